@@ -2,8 +2,7 @@
 // exact integer products and dequantization as the GEMMs (App. A / App. B.3
 // of the paper: per-token INT4 activations, per-output-channel INT4 weights,
 // acc = sum_k a_k w_k exact, y = fp16_rne((float(acc) * s_a) * s_w)), for
-// M <= 8 rows, where the weights are read once and the tensor cores would
-// sit idle: the cost is streaming the packed weights from HBM.
+// M <= 2 rows, where the cost is streaming the packed weights from HBM.
 //
 // Kernel: the M activation rows are sign-extended once into shared memory,
 // one byte per code (for each packed 32-bit word: its four low-nibble codes,
@@ -23,7 +22,7 @@ namespace p4q {
 namespace {
 
 constexpr int kGemvWarps = 8;
-constexpr int kGemvMaxRows = 8;  // above, the dp4a work per weight byte outweighs the stream
+constexpr int kGemvMaxRows = 2;  // above, the tensor-core kernel (p4q_fewrows.cu) is faster: 4 x 11008 x 4096 16.6 us here, 10.4 there
 constexpr int kGemvUnroll = 4;                  // weight chunks in flight per lane
 constexpr size_t kGemvSmemMax = 200u * 1024u;   // sign-extended activation rows
 
@@ -142,13 +141,6 @@ cudaError_t launch_mr(const GemmArgs& g, cudaStream_t stream) {
                     g.K, g.B, g.s_b, g.N, g.D);
 }
 
-template <bool S32>
-cudaError_t launch_rows(const GemmArgs& g, cudaStream_t stream) {
-  if (g.M <= 2) return launch_mr<2, S32>(g, stream);
-  if (g.M <= 4) return launch_mr<4, S32>(g, stream);
-  return launch_mr<8, S32>(g, stream);
-}
-
 }  // namespace
 
 bool gemv_applies(const GemmArgs& g) {
@@ -157,7 +149,7 @@ bool gemv_applies(const GemmArgs& g) {
 }
 
 cudaError_t launch_gemv(const GemmArgs& g, cudaStream_t stream) {
-  return g.out == GemmOut::kS32 ? launch_rows<true>(g, stream) : launch_rows<false>(g, stream);
+  return g.out == GemmOut::kS32 ? launch_mr<kGemvMaxRows, true>(g, stream) : launch_mr<kGemvMaxRows, false>(g, stream);
 }
 
 }  // namespace p4q
