@@ -148,6 +148,34 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   return __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
 }
 
+// One thread of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(pred));
+  return pred != 0;
+}
+
+// Bounded wait of a whole converged warp: every lane tests the barrier (no
+// divergent region around the test) and may sleep in hardware until the phase
+// completes, so that waiting warps leave the issue slots to working ones.
+__device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, volatile int* abort, unsigned int* err) {
+  const uint32_t a = smem_u32(bar);
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(a, parity))) return true;
+  const unsigned long long t0 = globaltimer();
+  while (true) {
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait_sleep(a, parity, 200000u))) return true;
+    if (__any_sync(0xFFFFFFFFu, *abort)) return false;
+    if (__any_sync(0xFFFFFFFFu, globaltimer() - t0 > kWaitLimitNs)) {
+      if ((threadIdx.x & 31) == 0) {
+        *abort = 1;
+        atomicOr(err, kErrTimeout);
+      }
+      __syncwarp();
+      return false;
+    }
+  }
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -203,6 +231,20 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint3
 // Barrier over `nthreads` threads (a multiple of 32) under the named barrier `id` (1..15).
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// named_bar_sync that also returns whether `pred` holds for any of the threads.
+__device__ __forceinline__ bool named_bar_or(uint32_t id, uint32_t nthreads, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"(id), "r"(nthreads), "r"(pred ? 1u : 0u)
+      : "memory");
+  return r != 0;
 }
 
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }

@@ -122,21 +122,6 @@ __device__ __forceinline__ void mma_f8f6f4_ts(uint32_t d_tmem, uint32_t a_tmem, 
       : "memory");
 }
 
-// One thread of a converged warp (the same one each time).
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(pred));
-  return pred != 0;
-}
-
-// Bounded wait of a whole converged warp, every lane testing the barrier (no
-// divergent region around the test).
-__device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, volatile int* abort, unsigned int* err) {
-  const uint32_t a = smem_u32(bar);
-  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(a, parity))) return true;
-  return mbar_wait_spin_warp(bar, parity, abort, err);
-}
-
 __device__ __forceinline__ float2 ld_shared_cluster_f32x2(uint32_t cluster_saddr) {
   float2 v;
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_saddr) : "memory");

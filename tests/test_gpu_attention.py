@@ -111,3 +111,13 @@ def test_attention_longest_sample(p4q, dev):
     q, k, v = _inputs(B, m, H, Hkv, seed=41)
     got = _run(p4q, dev, q, k, v, B, m, H, Hkv)
     _check(got, oracle.causal_attention(q, k, v, B, m, H, Hkv, DH), v, B, m, H, Hkv)
+
+
+@pytest.mark.parametrize("B,m,H,Hkv,scale", [(30, 100, 40, 40, 1.0), (3, 1000, 40, 8, 6.0), (20, 129, 32, 8, 3.0)])
+def test_attention_units_and_moving_maxima(p4q, dev, B, m, H, Hkv, scale):
+    """Several units per CTA of one chunk each, of mixed length, and of one and
+    two chunks, with row maxima that move past a unit's first chunk: the quads
+    of softmax warps run up to a chunk apart and the output staging is reused."""
+    q, k, v = _inputs(B, m, H, Hkv, seed=m, qscale=scale)
+    got = _run(p4q, dev, q, k, v, B, m, H, Hkv)
+    _check(got, oracle.causal_attention(q, k, v, B, m, H, Hkv, DH), v, B, m, H, Hkv)
