@@ -95,3 +95,17 @@ def test_swiglu_quant_column_blocks_without_expanded(p4q, dev):
     g, u = Y[:, 512:512 + K], Y[:, 512 + K:512 + 2 * K]
     _check(p4q, dev, np.ascontiguousarray(g), np.ascontiguousarray(u), expanded=False,
            G=Yd[:, 512:512 + K], U=Yd[:, 512 + K:512 + 2 * K])
+
+
+@pytest.mark.parametrize("M,K", [(610, 4112), (609, 6144), (609, 6160), (612, 12288), (612, 15360), (610, 15376),
+                                 (608, 4096), (3, 4112), (3, 12304)])
+def test_swiglu_quant_widths(p4q, dev, M, K):
+    """Row widths around what the CTA shapes hold (256 / 384 / 512 threads),
+    just above and below the row count from which the narrower ones run; some
+    chunks with gates past the two-at-a-time form's range (|g| > 87)."""
+    rng = np.random.default_rng(M + K)
+    g = (rng.standard_normal((M, K)) * 4).astype(np.float16)
+    u = (rng.standard_normal((M, K)) * 2).astype(np.float16)
+    at = rng.integers(0, K, M)
+    g[np.arange(M), at] = rng.choice(np.array([-500.0, -90.0, -88.0, -87.0, 87.0, 87.06, 88.0, 300.0]), M)
+    _check(p4q, dev, g, u)
