@@ -20,15 +20,24 @@
 // thread adds the bit patterns in four 32-bit words and turns them into one
 // 128-bit integer count of 2^-48 at the end.
 //
-// Kernel: one CTA per row, 128, 256 or 512 threads (so that a thread has at
-// most 4 chunks of 8 values, kept in registers); the block sums the 128-bit
-// integers (warp shuffles, then every thread adds the warp sums in warp
-// order), every thread forms r, then y, the row's abs-max (a second block
-// reduction) and the codes, written packed and, optionally, expanded one byte
-// per code (u = code + 8, the GEMM's order) with their row sum.
+// Kernel: one CTA per row, 128, 160, 256 or 512 threads (so that a thread has
+// at most 4 chunks of 8 values, kept in registers as fp16); a warp's four words
+// are added by integer reductions of their halfwords, every thread adds the
+// warps' sums into the 128-bit count and forms r, then y, the row's abs-max (a
+// second block reduction) and the codes, written packed and, optionally,
+// expanded one byte per code (u = code + 8, the GEMM's order) with their row
+// sum.
+//
+// Bound: instruction issue. The splits run two values at a time
+// (add/fma.rn.f32x2), t w is one fp16 multiplication (its exact product
+// rounded once, as the fp32 product rounded to fp16 is), the maxima are taken
+// on fp16 pairs and the codes from the bracketing products of p4q_codes.cuh.
+// Measured (us; one value at a time before): 2048 x 4096 9.4 (14.2) = 3.1 TB/s,
+// 2048 x 5120 13.0 (21.3), 16000 x 5120 79 (149).
 #include <cuda_fp16.h>
 
 #include "p4q.h"
+#include "p4q_codes.cuh"
 #include "p4q_device.cuh"
 #include "p4q_internal.h"
 
@@ -41,20 +50,27 @@ __device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) 
 
 constexpr float kM1 = 0x1.8p+33f, kM2 = 0x1.8p+11f, kM3 = 0x1.8p-11f, kM4 = 0x1.8p-25f;
 
-// acc[i] += bits of (residual + M_i) for the four splits of q = x^2
-__device__ __forceinline__ void add_square(float x, uint32_t (&acc)[4]) {
-  const float q = __fmul_rn(x, x);
-  const float a1 = __fadd_rn(q, kM1);
-  const float r1 = __fsub_rn(q, __fsub_rn(a1, kM1));
-  const float a2 = __fadd_rn(r1, kM2);
-  const float r2 = __fsub_rn(r1, __fsub_rn(a2, kM2));
-  const float a3 = __fadd_rn(r2, kM3);
-  const float r3 = __fsub_rn(r2, __fsub_rn(a3, kM3));
-  const float a4 = __fadd_rn(r3, kM4);
-  acc[0] += __float_as_uint(a1);
-  acc[1] += __float_as_uint(a2);
-  acc[2] += __float_as_uint(a3);
-  acc[3] += __float_as_uint(a4);
+// acc[i] += bits of (residual + M_i) for the four splits of the two squares q = x^2
+__device__ __forceinline__ void add_squares(float2 x, uint32_t (&acc)[4]) {
+  auto two = [](float c) { return make_float2(c, c); };
+  const float2 q = __fmul2_rn(x, x);
+  const float2 a1 = __fadd2_rn(q, two(kM1));
+  const float2 r1 = __ffma2_rn(__fadd2_rn(a1, two(-kM1)), two(-1.0f), q);  // q - (a1 - M1), exact
+  const float2 a2 = __fadd2_rn(r1, two(kM2));
+  const float2 r2 = __ffma2_rn(__fadd2_rn(a2, two(-kM2)), two(-1.0f), r1);
+  const float2 a3 = __fadd2_rn(r2, two(kM3));
+  const float2 r3 = __ffma2_rn(__fadd2_rn(a3, two(-kM3)), two(-1.0f), r2);
+  const float2 a4 = __fadd2_rn(r3, two(kM4));
+  acc[0] += __float_as_uint(a1.x) + __float_as_uint(a1.y);
+  acc[1] += __float_as_uint(a2.x) + __float_as_uint(a2.y);
+  acc[2] += __float_as_uint(a3.x) + __float_as_uint(a3.y);
+  acc[3] += __float_as_uint(a4.x) + __float_as_uint(a4.y);
+}
+
+// The warp's sum of the integers h (|h| < 2^31), by halfwords.
+__device__ __forceinline__ long long warp_sum(int h) {
+  const int lo = __reduce_add_sync(0xFFFFFFFFu, h & 0xFFFF), hi = __reduce_add_sync(0xFFFFFFFFu, h >> 16);
+  return static_cast<long long>(hi) * 65536 + lo;
 }
 
 __device__ __forceinline__ void add128(uint64_t& lo, uint64_t& hi, uint64_t lo2, uint64_t hi2) {
@@ -62,22 +78,13 @@ __device__ __forceinline__ void add128(uint64_t& lo, uint64_t& hi, uint64_t lo2,
   hi += hi2 + (lo < lo2 ? 1ull : 0ull);
 }
 
-__device__ __forceinline__ void add128s(uint64_t& lo, uint64_t& hi, long long v) {
-  add128(lo, hi, static_cast<uint64_t>(v), v < 0 ? ~0ull : 0ull);
-}
-
-// The thread's sum of squares as a 128-bit count of 2^-48 from the four words
-// (each holds n values' bits: n times the bits of M_i plus the sum of the H_i).
-__device__ __forceinline__ void acc_to_u128(const uint32_t (&acc)[4], int n, uint64_t& lo, uint64_t& hi) {
-  const long long h1 = static_cast<int>(acc[0] - static_cast<uint32_t>(n) * __float_as_uint(kM1));
-  const long long h2 = static_cast<int>(acc[1] - static_cast<uint32_t>(n) * __float_as_uint(kM2));
-  const long long h3 = static_cast<int>(acc[2] - static_cast<uint32_t>(n) * __float_as_uint(kM3));
-  const long long h4 = static_cast<int>(acc[3] - static_cast<uint32_t>(n) * __float_as_uint(kM4));
-  lo = static_cast<uint64_t>(h1) << 58;  // h1 >= 0, below 2^27
-  hi = static_cast<uint64_t>(h1) >> 6;
-  add128s(lo, hi, h2 * (1ll << 36));
-  add128s(lo, hi, h3 * (1ll << 14));
-  add128s(lo, hi, h4);
+// H1 2^58 + H2 2^36 + H3 2^14 + H4 (the count of 2^-48) as a 128-bit integer.
+__device__ __forceinline__ void splits_to_u128(const long long (&h)[4], uint64_t& lo, uint64_t& hi) {
+  lo = static_cast<uint64_t>(h[0]) << 58;  // h[0] >= 0
+  hi = static_cast<uint64_t>(h[0]) >> 6;
+  add128(lo, hi, static_cast<uint64_t>(h[1]) << 36, static_cast<uint64_t>(h[1] >> 28));
+  add128(lo, hi, static_cast<uint64_t>(h[2]) << 14, static_cast<uint64_t>(h[2] >> 50));
+  add128(lo, hi, static_cast<uint64_t>(h[3]), static_cast<uint64_t>(h[3] >> 63));
 }
 
 // fl32(S * 2^-48) for S = hi * 2^64 + lo, hi < 2^30: the top 64 bits of S with
@@ -99,8 +106,8 @@ __global__ void __launch_bounds__(THREADS)
   pdl_wait();
   pdl_launch_dependents();
   constexpr int kWarps = THREADS / 32;
-  __shared__ unsigned long long slo[kWarps], shi[kWarps];
-  __shared__ float wmax[kWarps];
+  __shared__ long long sh[kWarps][4];
+  __shared__ uint32_t wmax[kWarps];
   __shared__ int wsum[kWarps];
   const int row = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int nch = K >> 3;
@@ -118,79 +125,69 @@ __global__ void __launch_bounds__(THREADS)
   for (int j = 0; j < MAXC; ++j) {
     const uint32_t xw[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 xf = __half22float2(*reinterpret_cast<const __half2*>(&xw[e]));
-      add_square(xf.x, acc);
-      add_square(xf.y, acc);
-    }
+    for (int e = 0; e < 4; ++e) add_squares(__half22float2(*reinterpret_cast<const __half2*>(&xw[e])), acc);
   }
-  uint64_t lo, hi;
-  acc_to_u128(acc, 8 * MAXC, lo, hi);
+  // each word holds 8 MAXC values' bits: as many times the bits of M_i plus the sum of the H_i
+  const float kM[4] = {kM1, kM2, kM3, kM4};
+  long long h[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t lo2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), hi2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-    add128(lo, hi, lo2, hi2);
-  }
+  for (int i = 0; i < 4; ++i) h[i] = warp_sum(static_cast<int>(acc[i] - 8u * MAXC * __float_as_uint(kM[i])));
   if (lane == 0) {
-    slo[warp] = lo;
-    shi[warp] = hi;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sh[warp][i] = h[i];
   }
   __syncthreads();
-  lo = slo[0];
-  hi = shi[0];
 #pragma unroll
-  for (int v = 1; v < kWarps; ++v) add128(lo, hi, slo[v], shi[v]);
+  for (int i = 0; i < 4; ++i) {
+    h[i] = sh[0][i];
+#pragma unroll
+    for (int v = 1; v < kWarps; ++v) h[i] += sh[v][i];
+  }
+  uint64_t lo, hi;
+  splits_to_u128(h, lo, hi);
   const float ms = __fdiv_rn(sum_to_f32(lo, hi), static_cast<float>(K));
   const float den = __fadd_rn(ms, eps);
   const float r = den == 0.0f ? 0.0f : __frcp_rn(__fsqrt_rn(den));
-  // y = fp16(fp16(x * r) * w), kept as fp32 values
-  float y[MAXC][8];
-  float m = 0.0f;
+  // y = fp16(fp16(x * r) * w), in place of x
+  const float2 r2 = make_float2(r, r);
+  uint32_t m = 0;  // per-halfword max of |y| bit patterns
 #pragma unroll
   for (int j = 0; j < MAXC; ++j) {
     const int c = t + j * THREADS;
     const uint4 wv = c < nch ? __ldg(w4 + c) : make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t xw[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w}, ww[4] = {wv.x, wv.y, wv.z, wv.w};
+    uint32_t xw[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
+    const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float2 xf = __half22float2(*reinterpret_cast<const __half2*>(&xw[e]));
-      const float2 wf = __half22float2(*reinterpret_cast<const __half2*>(&ww[e]));
-      const float t0 = __half2float(__float2half_rn(__fmul_rn(xf.x, r)));
-      const float t1 = __half2float(__float2half_rn(__fmul_rn(xf.y, r)));
-      y[j][2 * e] = __half2float(__float2half_rn(__fmul_rn(t0, wf.x)));
-      y[j][2 * e + 1] = __half2float(__float2half_rn(__fmul_rn(t1, wf.y)));
-      m = fmaxf(m, fmaxf(fabsf(y[j][2 * e]), fabsf(y[j][2 * e + 1])));
+      const float2 tf = __fmul2_rn(__half22float2(*reinterpret_cast<const __half2*>(&xw[e])), r2);
+      const __half2 y = __hmul2_rn(__floats2half2_rn(tf.x, tf.y), *reinterpret_cast<const __half2*>(&ww[e]));
+      xw[e] = *reinterpret_cast<const uint32_t*>(&y);
+      m = __vmaxu2(m, xw[e] & 0x7FFF7FFFu);
     }
+    xv[j] = make_uint4(xw[0], xw[1], xw[2], xw[3]);
   }
-  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 16));
-  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 8));
-  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 4));
-  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-  if (lane == 0) wmax[warp] = m;
+  const uint32_t wm = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+  if (lane == 0) wmax[warp] = wm;
   __syncthreads();
-  float a = 0.0f;
+  uint32_t am = wmax[0];
 #pragma unroll
-  for (int v = 0; v < kWarps; ++v) a = fmaxf(a, wmax[v]);
-  const float s = __fdiv_rn(a, 7.0f);
-  const float inv = (a != 0.0f) ? __frcp_rn(s) : 0.0f;
+  for (int v = 1; v < kWarps; ++v) am = max(am, wmax[v]);
+  const float a = __half2float(__ushort_as_half(static_cast<unsigned short>(am)));
+  const QRow q = quant_row(a);
+  const float s = q.s;
   uint32_t* q4 = reinterpret_cast<uint32_t*>(Xq + static_cast<size_t>(row) * (K >> 1));
   uint2* up2 = EXPANDED ? reinterpret_cast<uint2*>(Xu + static_cast<size_t>(row) * K) : nullptr;
   uint32_t su = 0;
+  float2 n2 = make_float2(0.0f, 0.0f);  // unused
 #pragma unroll
   for (int j = 0; j < MAXC; ++j) {
     const int c = t + j * THREADS;
     if (c < nch) {
-      // value e of the chunk in bits 4e: byte i holds values 2i (low nibble) and 2i + 1
-      uint32_t pw = 0;
-      if (a != 0.0f) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) pw |= (static_cast<uint32_t>(q4_code(y[j][e], s, inv)) & 0xFu) << (4 * e);
-      }
-      q4[c] = pw;
+      const Codes8 cd = (a != 0.0f) ? quant_chunk<false>(xv[j], q, n2) : Codes8{0u, 0u};
+      q4[c] = packed4(cd);
       if (EXPANDED) {
         // the even values, then the odd ones, offset by 8 (the GEMM's order)
-        const uint32_t eu = (pw & 0x0F0F0F0Fu) ^ 0x08080808u, ou = ((pw >> 4) & 0x0F0F0F0Fu) ^ 0x08080808u;
+        const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
         up2[c] = make_uint2(eu, ou);
         su = __dp4a(eu + ou, 0x01010101u, su);
       }
@@ -239,6 +236,7 @@ cudaError_t launch_rmsnorm_quant(const uint16_t* X16, long long ldx, const uint1
   const __half* w = reinterpret_cast<const __half*>(w16);
   static_assert(P4Q_MAX_ROW <= 8 * 512 * kRnMaxChunks, "rows longer than 512 threads x 4 chunks");
   if (K <= 8 * 128 * kRnMaxChunks) return launch_t<128>(X, ldx, w, eps, M, K, Xq, s_a, Xu, sum_xu, stream);
+  if (K <= 8 * 160 * kRnMaxChunks) return launch_t<160>(X, ldx, w, eps, M, K, Xq, s_a, Xu, sum_xu, stream);
   if (K <= 8 * 256 * kRnMaxChunks) return launch_t<256>(X, ldx, w, eps, M, K, Xq, s_a, Xu, sum_xu, stream);
   return launch_t<512>(X, ldx, w, eps, M, K, Xq, s_a, Xu, sum_xu, stream);
 }

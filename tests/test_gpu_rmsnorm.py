@@ -78,3 +78,13 @@ def test_rmsnorm_quant_row_pitch_without_expanded(p4q, dev):
     Yd = torch.from_numpy(Y).to(dev)
     w = (1.0 + 0.1 * rng.standard_normal(K)).astype(np.float16)
     _check(p4q, dev, np.ascontiguousarray(Y[:, 1024:1024 + K]), w, 1e-6, expanded=False, X=Yd[:, 1024:1024 + K])
+
+
+@pytest.mark.parametrize("M,K", [(2, 1040), (3, 4112), (4, 5120), (3, 5136), (2, 8192), (2, 8208), (700, 2048)])
+def test_rmsnorm_quant_widths(p4q, dev, M, K):
+    """Row widths around what the CTA shapes hold (128 / 160 / 256 / 512
+    threads of up to four chunks), values over the whole fp16 range."""
+    rng = np.random.default_rng(M + K)
+    x = (rng.standard_normal((M, K)) * 2.0 ** rng.integers(-20, 14, (M, K))).astype(np.float16)
+    w = (1.0 + 0.5 * rng.standard_normal(K)).astype(np.float16)
+    _check(p4q, dev, x, w, 1e-6)
