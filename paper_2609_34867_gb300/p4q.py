@@ -107,14 +107,20 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+# Pointers and streams go to ctypes as plain integers (the argtypes make them
+# void pointers), and the current stream is asked for as its raw handle: a
+# torch.cuda.Stream object for it takes 2.8 us, a third of a short call
+# (p4q_quant_act on 8 rows 8.2 -> 4.1 us of host time).
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _check(status: int, what: str):
