@@ -296,6 +296,7 @@ p4q_status p4q_quant_act_expanded(const uint16_t* X, int ldx, int M, int Kin, ui
   RowSource src;
   src.X = X;
   src.ldx = ldx;
+  src.early = true;
   RowSinks o;
   o.codes = Xq;
   o.scale = s_a;
@@ -396,6 +397,7 @@ p4q_status p4q_quant_act_ld(const uint16_t* X, int ldx, int M, int Kin, uint8_t*
   RowSource src;
   src.X = X;
   src.ldx = ldx;
+  src.early = true;
   RowSinks o;
   o.codes = Xq;
   o.scale = s_a;

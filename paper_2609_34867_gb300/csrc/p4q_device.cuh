@@ -31,6 +31,12 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 // serialization: it may start while the previous kernel on the stream is
 // finishing, does only private setup (shared memory, barriers, TMEM) before
 // pdl_wait(), and lets the next kernel launch as soon as it has passed it.
+// The quantizers in front of the linears, and the linears that prefetch their
+// weights into L2 before their wait, let it launch before their own wait (and
+// after any TMEM allocation): a kernel's wait ends when the one before it has
+// completed, which that one does only after its own wait, so what a kernel
+// reads is still complete; and the weights of a linear are on their way while
+// the linear before its quantizer still runs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

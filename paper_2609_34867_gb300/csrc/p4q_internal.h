@@ -41,6 +41,9 @@ struct RowSource {
   int N = 0, K = 0, T = 0;         // gather mode sizes
   const uint16_t* X2 = nullptr;    // dense rows split, split + 1, ... (the second sinks; dense mode)
   int split = 0;
+  // lets the next kernel launch before this one's wait (a linear that prefetches its
+  // weights meanwhile); in the selector's chain that made calls 3% slower
+  bool early = false;
 };
 
 // Outputs of the per-row quantizer. Optional pointers may be null.

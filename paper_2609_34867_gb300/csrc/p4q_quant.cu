@@ -88,8 +88,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   if (threadIdx.x < kGroups) aborts[threadIdx.x] = 0;
   fence_barrier_init();
   __syncthreads();
+  if (src.early) pdl_launch_dependents();
   pdl_wait();  // rows (and kept indices) come from the previous kernel
-  pdl_launch_dependents();
+  if (!src.early) pdl_launch_dependents();
 
   unsigned char* ring = smem + static_cast<size_t>(grp) * S * stage_bytes;
   uint64_t* full = bars + grp * S;

@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(THREADS)
     rmsnorm_quant_kernel(const __half* __restrict__ X, long long ldx, const __half* __restrict__ w, float eps, int K,
                          uint8_t* __restrict__ Xq, float* __restrict__ s_a, uint8_t* __restrict__ Xu,
                          int32_t* __restrict__ sum_xu) {
+  pdl_launch_dependents();  // before the wait: see p4q_device.cuh
   pdl_wait();
-  pdl_launch_dependents();
   constexpr int kWarps = THREADS / 32;
   __shared__ long long sh[kWarps][4];
   __shared__ uint32_t wmax[kWarps];

@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (MAXC <= 3 ? 4 : 2) 
     swiglu_quant_kernel(const __half* __restrict__ gate, long long ldg, const __half* __restrict__ up, long long ldu,
                         int K, uint8_t* __restrict__ Xq, float* __restrict__ s_a, uint8_t* __restrict__ Xu,
                         int32_t* __restrict__ sum_xu) {
+  pdl_launch_dependents();  // before the wait: see p4q_device.cuh
   pdl_wait();
-  pdl_launch_dependents();
   __shared__ float wmax[THREADS / 32];
   __shared__ int wsum[THREADS / 32];
   const int row = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
