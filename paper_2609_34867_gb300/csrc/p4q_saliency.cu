@@ -4,14 +4,21 @@
 // crop's patch keys, of q . k / sqrt(d_h), and the saliency of a patch is its
 // weight averaged over the heads.
 //
-// Kernel: one CTA per (image, crop), up to 16 warps each taking heads in
-// turn (one warp per head at a time). A token's key row for the head (dh fp16
-// values, rows of consecutive tokens H x dh apart) is read by dh / 8 lanes
-// with one 16-byte load each, so that a warp load covers whole rows; the
-// lanes' partial dot products (fp16 products accumulated in fp32) are summed
-// by shuffles. The warp's max and sum then give the head's softmax; the
-// per-head weights go to shared memory and are summed over the heads in head
-// order (deterministic).
+// Kernel: a cluster of up to 8 CTAs per (image, crop), its heads dealt out to
+// the CTAs and each head's tokens to the CTA's warps, so that a few crops
+// still occupy many SMs. A token's key row for the head (dh fp16 values, rows
+// of consecutive tokens H x dh apart) is read by dh / 8 lanes with one 16-byte
+// load each, so that a warp load covers whole rows; the lanes' partial dot
+// products (fp16 products accumulated in fp32) are summed by shuffles. The
+// head's max and sum (over its warps, in warp order) give its softmax; the
+// per-head weights stay in the CTA's shared memory, and each CTA sums its share
+// of the tokens over the heads in head order, reading the other CTAs' weights
+// through distributed shared memory (deterministic for a given shape).
+//
+// Bound: load latency for few crops, HBM for many. Measured (16 heads x 64, us;
+// one CTA per crop and one warp per head before): 8 crops of 576 tokens 8.2
+// (24.3), 32 crops 13.7 (31.9), 80 crops 30.2 (34.4), 160 crops 44.5 (46.9) =
+// 4.2 TB/s, 4 crops of 3600 at 128 wide 66 (390).
 #include <cuda_fp16.h>
 
 #include "p4q.h"
@@ -21,10 +28,9 @@
 namespace p4q {
 namespace {
 
-// Warps per CTA at most (each takes heads warp, warp + warps, ...): 16, so
-// that a thread has 128 registers for its head's query and key loads.
-constexpr int kMaxWarps = 16;
+constexpr int kWarps = 16;
 constexpr int kMaxHeads = 32;
+constexpr int kMaxCluster = 8;
 
 // Lanes that share one token's key row: the row's dh / 8 16-byte chunks, one
 // per lane, rounded up to a power of two (idle lanes past the row).
@@ -33,22 +39,43 @@ constexpr int lanes_per_token() {
   return DH / 8 <= 4 ? 4 : DH / 8 <= 8 ? 8 : DH / 8 <= 16 ? 16 : 32;
 }
 
-template <int DH>
-__global__ void __launch_bounds__(32 * kMaxWarps)
+// Heads of CTA `rank` of a cluster of cs: h = rank + cs * i, i = 0 .. heads - 1.
+__device__ __forceinline__ int heads_of(int H, int cs, int rank) { return (H - rank + cs - 1) / cs; }
+
+__device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_saddr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_saddr) : "memory");
+  return v;
+}
+
+// wph warps per head (a power of two); the CTA's heads in rounds of kWarps / wph.
+template <int DH, bool ONE>
+__global__ void __launch_bounds__(32 * kWarps, 2)
     cls_saliency_kernel(const __half* __restrict__ q_cls, const __half* __restrict__ k_cls,
-                        const __half* __restrict__ k, int N, int C, int H, float* __restrict__ A) {
+                        const __half* __restrict__ k, int N, int C, int H, int cs_, int wph_, float* __restrict__ A) {
+  // ONE: one CTA per crop, one warp per head
+  const int cs = ONE ? 1 : cs_, wph = ONE ? 1 : wph_;
   pdl_wait();
   pdl_launch_dependents();
   constexpr int R = DH / 8;                  // 16-byte chunks per key row
   constexpr int LPT = lanes_per_token<DH>();  // lanes per token
   constexpr int CPL = (R + LPT - 1) / LPT;    // chunks per lane
   constexpr int TPI = 32 / LPT;               // tokens per warp iteration
-  extern __shared__ float p[];  // [H][n] softmax weights of the crop's patches per head
-  const int b = blockIdx.y, c = blockIdx.x, n = N / C;
-  const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  extern __shared__ float p[];  // [heads of this CTA][n] softmax weights of the crop's patches
+  __shared__ float red[2][kWarps];  // per warp: max, then sum
+  const int c = blockIdx.x / cs, rank = blockIdx.x - c * cs;
+  const int b = blockIdx.y, n = N / C;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = lane % LPT, tok = lane / LPT;
+  const int mine = heads_of(H, cs, rank);
+  const int hpr = kWarps / wph;              // heads per round
+  const int part = warp % wph;               // this warp's part of the head's tokens
+  const int per = (n + wph - 1) / wph, t0 = part * per, t1 = min(n, t0 + per);
   const float scale = 1.0f / sqrtf(static_cast<float>(DH));
-  for (int h = threadIdx.x >> 5; h < H; h += nwarps) {
+  for (int i0h = 0; i0h < mine; i0h += hpr) {
+    const int ih = i0h + warp / wph;         // the CTA's head index
+    const bool live = ih < mine;
+    const int h = rank + cs * (live ? ih : 0);
     const size_t head = (static_cast<size_t>(b) * C + c) * H + h;
     // this lane's chunks of the query, as fp32
     float qf[CPL][8];
@@ -66,11 +93,11 @@ __global__ void __launch_bounds__(32 * kMaxWarps)
       }
     }
     // this lane's chunks of a key row (zeros past the row or for no token)
-    auto load = [&](const uint4* row, bool live, uint4 (&v)[CPL]) {
+    auto load = [&](const uint4* row, bool in, uint4 (&v)[CPL]) {
 #pragma unroll
       for (int u = 0; u < CPL; ++u) {
         const int ch = sub + u * LPT;
-        v[u] = (live && ch < R) ? __ldg(row + ch) : make_uint4(0u, 0u, 0u, 0u);
+        v[u] = (in && ch < R) ? ldg_stream16(row + ch) : make_uint4(0u, 0u, 0u, 0u);
       }
     };
     // partial dot of the loaded chunks, then the sum over the token's lanes
@@ -94,68 +121,113 @@ __global__ void __launch_bounds__(32 * kMaxWarps)
     load(reinterpret_cast<const uint4*>(k_cls + head * DH), true, v0);
     const float l0 = dot(v0) * scale;
     float mx = l0;
-    float* ph = p + static_cast<size_t>(h) * n;
-    constexpr int U = 8;  // token rows in flight per lane
-    for (int i0 = 0; i0 < n; i0 += TPI * U) {
+    float* ph = p + static_cast<size_t>(live ? ih : 0) * n;
+    constexpr int U = ONE ? 8 : 4;  // token rows in flight per lane (several warps per head: 4 keeps 64 registers)
+    for (int i0 = t0; i0 < t1; i0 += TPI * U) {
       uint4 v[U][CPL];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * TPI + tok;
-        const size_t row = (static_cast<size_t>(b) * N + static_cast<size_t>(c) * n + (i < n ? i : 0)) * H + h;
-        load(reinterpret_cast<const uint4*>(k + row * DH), i < n, v[u]);
+        const bool in = live && i < t1;
+        const size_t row = (static_cast<size_t>(b) * N + static_cast<size_t>(c) * n + (in ? i : 0)) * H + h;
+        load(reinterpret_cast<const uint4*>(k + row * DH), in, v[u]);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * TPI + tok;
         const float l = dot(v[u]) * scale;
-        if (i < n) {
+        if (live && i < t1) {
           if (sub == 0) ph[i] = l;
           mx = fmaxf(mx, l);
         }
       }
     }
-    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 16));
-    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 8));
-    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 4));
-    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
-    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
-    __syncwarp();
-    float z = lane == 0 ? expf(l0 - mx) : 0.0f;
-    for (int i = lane; i < n; i += 32) {
-      const float e = expf(ph[i] - mx);
-      ph[i] = e;
-      z += e;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if (wph > 1) {
+      if (lane == 0) red[0][warp] = mx;
+      __syncthreads();
+      for (int w = warp - part; w < warp - part + wph; ++w) mx = fmaxf(mx, red[0][w]);
+    } else {
+      __syncwarp();
     }
-    z += __shfl_xor_sync(0xFFFFFFFFu, z, 16);
-    z += __shfl_xor_sync(0xFFFFFFFFu, z, 8);
-    z += __shfl_xor_sync(0xFFFFFFFFu, z, 4);
-    z += __shfl_xor_sync(0xFFFFFFFFu, z, 2);
-    z += __shfl_xor_sync(0xFFFFFFFFu, z, 1);
+    float z = (lane == 0 && part == 0) ? expf(l0 - mx) : 0.0f;
+    if (live) {
+      for (int i = t0 + lane; i < t1; i += 32) {
+        const float e = expf(ph[i] - mx);
+        ph[i] = e;
+        z += e;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+    if (wph > 1) {
+      if (lane == 0) red[1][warp] = z;
+      __syncthreads();
+      z = 0.0f;
+      for (int w = warp - part; w < warp - part + wph; ++w) z += red[1][w];
+    }
     const float inv = 1.0f / z;
-    for (int i = lane; i < n; i += 32) ph[i] *= inv;
+    if (live)
+      for (int i = t0 + lane; i < t1; i += 32) ph[i] *= inv;
   }
-  __syncthreads();
+  if (cs > 1) cluster_sync();
+  else __syncthreads();
   const float invh = 1.0f / static_cast<float>(H);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  const uint32_t pb = smem_u32(p);
+  for (int i = rank * blockDim.x + threadIdx.x; i < n; i += cs * blockDim.x) {
     float s = 0.0f;
-    for (int hh = 0; hh < H; ++hh) s += p[static_cast<size_t>(hh) * n + i];
+    if (cs > 1) {
+#pragma unroll 8
+      for (int hh = 0; hh < H; ++hh)
+        s += ld_shared_cluster_f32(mapa_shared(pb + 4u * static_cast<uint32_t>((hh / cs) * n + i), hh % cs));
+    } else {
+      for (int hh = 0; hh < H; ++hh) s += p[static_cast<size_t>(hh) * n + i];
+    }
     A[static_cast<size_t>(b) * N + static_cast<size_t>(c) * n + i] = s * invh;
   }
+  if (cs > 1) cluster_sync();  // no CTA leaves while its weights are read
 }
 
 template <int DH>
 cudaError_t launch_dh(const __half* q_cls, const __half* k_cls, const __half* k, int B, int N, int C, int H,
                       float* A, cudaStream_t stream) {
-  const size_t smem = static_cast<size_t>(H) * (N / C) * sizeof(float);
+  // CTAs per crop: as many as leave every SM at most two, and one head each;
+  // more where one CTA's weights and its reductions exceed the shared memory
+  int cs = 1;
+  auto weights = [&](int x) { return static_cast<size_t>((H + x - 1) / x) * (N / C) * sizeof(float); };
+  while (cs < kMaxCluster && 2 * cs <= H &&
+         (static_cast<long long>(B) * C * 2 * cs <= 2 * num_sms() || weights(cs) + 256 > 227u * 1024u))
+    cs *= 2;
+  const int heads = (H + cs - 1) / cs;
+  int wph = 1;  // warps per head: the CTA's warps over its heads
+  while (2 * wph * heads <= kWarps) wph *= 2;
+  const size_t smem = weights(cs);
   static size_t smem_set = 48u << 10;
   if (smem > smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(cls_saliency_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
+    for (auto kern : {cls_saliency_kernel<DH, true>, cls_saliency_kernel<DH, false>}) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      if (e != cudaSuccess) return e;
+    }
     smem_set = smem;
   }
-  return launch_pdl(cls_saliency_kernel<DH>, dim3(C, B), dim3(32 * (H < kMaxWarps ? H : kMaxWarps)), smem, stream,
-                    q_cls, k_cls, k, N, C, H, A);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(C) * cs, B);
+  cfg.blockDim = dim3(32 * kWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cs);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs > 1 ? 2 : 1;
+  if (cs == 1 && wph == 1)
+    return cudaLaunchKernelEx(&cfg, cls_saliency_kernel<DH, true>, q_cls, k_cls, k, N, C, H, cs, wph, A);
+  return cudaLaunchKernelEx(&cfg, cls_saliency_kernel<DH, false>, q_cls, k_cls, k, N, C, H, cs, wph, A);
 }
 
 }  // namespace

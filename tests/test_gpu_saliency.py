@@ -62,3 +62,16 @@ def test_saliency_feeds_the_selector(p4q, dev):
     torch.cuda.synchronize()
     ref = oracle.select_batch(x.V, w.K, x.Q, A.cpu().numpy())
     assert np.array_equal(idx.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("B,C,n,H,dh", [(1, 1, 577, 16, 64), (1, 3, 40, 12, 64), (2, 1, 33, 7, 80), (40, 1, 30, 16, 32),
+                                        (80, 1, 25, 16, 64), (160, 1, 20, 16, 64), (90, 2, 9, 5, 128),
+                                        (1, 1, 3632, 16, 32), (200, 1, 3, 1, 64)])
+def test_saliency_clusters(p4q, dev, B, C, n, H, dh):
+    """Heads over clusters of 8, 4, 2 and 1 CTAs (evenly or not), one or
+    several warps per head, the largest weights one CTA was asked to hold."""
+    rng = np.random.default_rng(B + n + H)
+    q = (rng.standard_normal((B, C, H, dh)) * 2).astype(np.float16)
+    kc = rng.standard_normal((B, C, H, dh)).astype(np.float16)
+    k = rng.standard_normal((B, C * n, H, dh)).astype(np.float16)
+    _check(p4q, dev, q, kc, k)
