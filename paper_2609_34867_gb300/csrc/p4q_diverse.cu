@@ -54,9 +54,7 @@ constexpr int kStageBytes = (kArows + kBrows) * kBK;
 constexpr uint32_t kTmemCols = 256;
 
 struct DivScratch {
-  unsigned int hist[256];
-  unsigned int wsum[32];
-  int digit, above;
+  RankScratch rank;
   int t, npool, tmin, nphase;
   unsigned long long tau;
   __align__(16) unsigned long long skey[kPool];  // pool rounds: (m, slot) keys of the certain entries
@@ -82,10 +80,6 @@ struct DivScratch {
   volatile int abort_flag;
   __align__(16) float cp[kPool][kPool + 1]; // cos(ptok[i], ptok[j]) (Eq. 4, exact; padded: column writes)
 };
-
-__device__ __forceinline__ float order_key_float(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
 
 // Greedy rounds on the pool, by the whole block (thread i < 128 owns pool
 // slot i), with exact m of the pool entries in s.pm. The next pick is the
@@ -262,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
         member[e] = kept[e];
         key[e] = (base + e < N) ? ~float_order_key(m[e]) : 0u;
       }
-      block_take_top(key, member, base, N, q, tpg, s);
+      block_take_top<true>(key, member, base, N, q, tpg, s.rank);
       int cnt = 0, emin = t;
 #pragma unroll
       for (int e = 0; e < kPer; ++e) {
@@ -270,7 +264,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
         cnt += in ? 1 : 0;
         emin = in ? min(emin, ex[e]) : emin;
       }
-      int pos = block_exclusive_scan(cnt, &npool, tpg, s);
+      group_sync(tpg);
+      int pos = block_exclusive_scan(cnt, &npool, tpg, s.rank);
 #pragma unroll
       for (int e = 0; e < kPer; ++e) {
         if (base + e < N && member[e] && !kept[e]) {
@@ -554,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     for (int e = 0; e < kPer; ++e)
       cnt += (base + e < N && ((s.keptbits[(base + e) >> 5] >> ((base + e) & 31)) & 1u)) ? 1 : 0;
     int total;
-    int pos = block_exclusive_scan(cnt, &total, tpg, s);
+    int pos = block_exclusive_scan(cnt, &total, tpg, s.rank);
 #pragma unroll
     for (int e = 0; e < kPer; ++e)
       if (base + e < N && ((s.keptbits[(base + e) >> 5] >> ((base + e) & 31)) & 1u) && pos < a.K)

@@ -10,7 +10,7 @@
 // evaluated on their codes (code_cosine: the positive per-row scales cancel).
 //
 // Kernels:
-//   select_stages12_kernel  one CTA per image, one thread per 4 tokens: stage 1
+//   select_stages12_kernel  one CTA per image, one thread per token (2 - 4 past 1024 tokens): stage 1
 //                           (per-concept top quota), stage 2 (CLS-saliency top
 //                           K_s); writes the kept set R0 as bits and as an
 //                           ascending token list (and as idx when K_d = 0).
@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "p4q.h"
 #include "p4q_device.cuh"
@@ -41,24 +42,20 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-// Upper bound on the stages-1/2 block: one thread per kPer tokens (N <= 4096).
+// Threads of a ranking block at most (N <= 4096: up to 4 tokens each).
 constexpr int kSelThreads = 1024;
 
-struct RankScratch {
-  unsigned int hist[256];
-  unsigned int wsum[32];
-  int digit, above;
-};
-
-// Stages 1 and 2 of Eq. 4 for image blockIdx.x, on blockDim.x = ceil(N / 4)
+// Stages 1 and 2 of Eq. 4 for image blockIdx.x, on blockDim.x = ceil(N / PER)
 // rounded up to a warp: query relevance (one ranking per concept, quota
 // floor(Kq / J) + (j < Kq % J), each concept keeps its best tokens not yet
 // kept), then visual saliency (the best Ks of A_cls among the rest). The kept
 // set R0 goes out as bits (token t: bit t % 32 of word t / 32 of the image's
 // row of kept12), as the ascending list r0tok [B, R0] (R0 = Kq + Ks), and as
-// idx when there is no diversity stage.
-template <int kMaxThreads>
-__global__ void __launch_bounds__(kMaxThreads, 1)
+// idx when there is no diversity stage. As many threads as tokens where the
+// block allows (PER = 1 up to 1024 tokens): an exact cosine is on the order of
+// a hundred instructions, and every load of the scores goes out first.
+template <int PER>
+__global__ void __launch_bounds__(kSelThreads, 1)
     select_stages12_kernel(const float* __restrict__ qdots, int qp, const int32_t* __restrict__ qnorm,
                            const int32_t* __restrict__ vnorm, const float* __restrict__ A_cls, int N, int J, int Kq,
                            int Ks, int Kd, uint32_t* __restrict__ kept12, int32_t* __restrict__ r0tok,
@@ -66,48 +63,65 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
   pdl_wait();
   pdl_launch_dependents();
   __shared__ RankScratch s;
+  __shared__ uint32_t bits[P4Q_MAX_TOKENS / 32];
   const int b = blockIdx.x, nt = blockDim.x;
-  const int base = kPer * threadIdx.x;
-  bool kept[kPer];
+  const int base = PER * threadIdx.x;
+  const int words = (N + 31) / 32;
+  for (int w = threadIdx.x; w < words; w += nt) bits[w] = 0;
+  bool kept[PER];
+  float acls[PER];
+  int nv[PER];  // squared code norms of the thread's tokens
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) kept[e] = false;
-  uint32_t key[kPer];
-  int nv[kPer];  // squared code norms of the thread's tokens
+  for (int e = 0; e < PER; ++e) {
+    const size_t t = static_cast<size_t>(b) * N + base + e;
+    const bool in = base + e < N;
+    kept[e] = false;
+    nv[e] = (Kq > 0 && in) ? vnorm[t] : 0;
+    acls[e] = (Ks > 0 && in) ? A_cls[t] : 0.0f;
+  }
+  uint32_t key[PER];
+  for (int j0 = 0; j0 < J && Kq > 0; j0 += 4) {
+    // Eq. 4 query cosines of each token with four concepts, from the exact dot products
+    float4 qd[PER];
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) nv[e] = (Kq > 0 && base + e < N) ? vnorm[static_cast<size_t>(b) * N + base + e] : 0;
-  for (int j = 0; j < J && Kq > 0; ++j) {
-    const int quota = Kq / J + (j < Kq % J ? 1 : 0);
-    const int nq = qnorm[b * J + j];
-    // Eq. 4 query cosine of each token with concept j, from the exact dot products
+    for (int e = 0; e < PER; ++e)
+      qd[e] = base + e < N
+                  ? *reinterpret_cast<const float4*>(qdots + (static_cast<size_t>(b) * N + base + e) * qp + j0)
+                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-      const size_t t = static_cast<size_t>(b) * N + base + e;
-      key[e] = (base + e < N) ? float_order_key(code_cosine(static_cast<int>(qdots[t * qp + j]), nq, nv[e])) : 0u;
+    for (int jj = 0; jj < 4; ++jj) {
+      const int j = j0 + jj;
+      if (j >= J) break;
+      const int quota = Kq / J + (j < Kq % J ? 1 : 0);
+      const int nq = qnorm[b * J + j];
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        const float dot = jj == 0 ? qd[e].x : jj == 1 ? qd[e].y : jj == 2 ? qd[e].z : qd[e].w;
+        key[e] = float_order_key(code_cosine(static_cast<int>(dot), nq, nv[e]));
+      }
+      block_take_top<false>(key, kept, base, N, quota, nt, s);
     }
-    block_take_top(key, kept, base, N, quota, nt, s);
   }
   if (Ks > 0) {
-    const float* a = A_cls + static_cast<size_t>(b) * N;
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) key[e] = (base + e < N) ? float_order_key(a[base + e]) : 0u;
-    block_take_top(key, kept, base, N, Ks, nt, s);
+    for (int e = 0; e < PER; ++e) key[e] = float_order_key(acls[e]);
+    block_take_top<false>(key, kept, base, N, Ks, nt, s);
   }
-  // kept bits: the four tokens of a thread share a word (kPer divides 32)
-  uint32_t bits = 0;
-#pragma unroll
-  for (int e = 0; e < kPer; ++e) bits |= (base + e < N && kept[e]) ? 1u << ((base + e) & 31) : 0u;
-  const unsigned word_peers = 0xFFu << (8 * ((threadIdx.x & 31) >> 3));  // the 8 lanes of one 32-token word
-  bits = __reduce_or_sync(word_peers, bits);
-  const int words = (N + 31) / 32;
-  if ((threadIdx.x & 7) == 0 && base / 32 < words) kept12[static_cast<size_t>(b) * words + base / 32] = bits;
+  group_sync(nt);  // the words are cleared (and the rankings done) before bits are set
   int cnt = 0;
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) cnt += (base + e < N && kept[e]) ? 1 : 0;
+  for (int e = 0; e < PER; ++e) {
+    if (base + e < N && kept[e]) {
+      ++cnt;
+      atomicOr(&bits[(base + e) >> 5], 1u << ((base + e) & 31));
+    }
+  }
   int total;
   int pos = block_exclusive_scan(cnt, &total, nt, s);
+  for (int w = threadIdx.x; w < words; w += nt) kept12[static_cast<size_t>(b) * words + w] = bits[w];
   const int R0 = Kq + Ks;
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) {
+  for (int e = 0; e < PER; ++e) {
     if (base + e < N && kept[e] && pos < R0) {
       r0tok[static_cast<size_t>(b) * R0 + pos] = base + e;
       if (Kd == 0) idx[static_cast<size_t>(b) * R0 + pos] = base + e;
@@ -121,48 +135,45 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 // R0, as an ascending list cand [B, C]. Greedy picks and pool entries are
 // taken among the smallest pairs and pairs only grow, so the stage usually
 // needs the cosines of candidates only (the GEMM over them); it checks, per
-// pool phase, that it does. Same layout and radix select as stages 1-2.
-template <int kMaxThreads>
-__global__ void __launch_bounds__(kMaxThreads, 1)
+// pool phase, that it does. Same layout and ranking as stages 1-2.
+template <int PER>
+__global__ void __launch_bounds__(kSelThreads, 1)
     select_candidates_kernel(float* __restrict__ m, const float* __restrict__ mpart, int parts,
                              const uint32_t* __restrict__ kept12, int N, int R0, int C, int32_t* __restrict__ cand) {
   pdl_wait();
   pdl_launch_dependents();
-  if (mpart != nullptr) {
-    // m = the largest of the per-column-tile maxima (stage 3 reads m too)
-    const size_t part = static_cast<size_t>(gridDim.x) * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const size_t t = static_cast<size_t>(blockIdx.x) * N + i;
-      float v = mpart[t];
-      for (int k = 1; k < parts; ++k) v = fmaxf(v, mpart[k * part + t]);
-      m[t] = v;
-    }
-    __syncthreads();
-  }
   __shared__ RankScratch s;
   const int b = blockIdx.x, nt = blockDim.x;
-  const int base = kPer * threadIdx.x;
+  const int base = PER * threadIdx.x;
   const int words = (N + 31) / 32;
-  bool taken[kPer];
-  uint32_t key[kPer];
+  const size_t part = static_cast<size_t>(gridDim.x) * N;
+  bool taken[PER], in_r0[PER];
+  uint32_t key[PER];
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) {
+  for (int e = 0; e < PER; ++e) {
     const int i = base + e;
+    const size_t t = static_cast<size_t>(b) * N + i;
     taken[e] = i < N && ((kept12[static_cast<size_t>(b) * words + (i >> 5)] >> (i & 31)) & 1u);
-    // the smallest pairs as the largest keys; m = -inf (R0 empty) ranks every token equal
-    key[e] = (i < N) ? ~float_order_key(R0 > 0 ? m[static_cast<size_t>(b) * N + i] : -INFINITY) : 0u;
+    in_r0[e] = taken[e];
+    float v = -INFINITY;  // m = -inf (R0 empty) ranks every token equal
+    if (i < N && mpart != nullptr) {
+      // m = the largest of the per-column-tile maxima (stage 3 reads m too)
+      for (int k = 0; k < parts; ++k) v = fmaxf(v, mpart[k * part + t]);
+      m[t] = v;
+    } else if (i < N && R0 > 0) {
+      v = m[t];
+    }
+    key[e] = ~float_order_key(v);  // the smallest pairs as the largest keys
   }
-  bool in_r0[kPer];
-#pragma unroll
-  for (int e = 0; e < kPer; ++e) in_r0[e] = taken[e];
-  block_take_top(key, taken, base, N, C, nt, s);
+  block_take_top<true>(key, taken, base, N, C, nt, s);
   int cnt = 0;
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) cnt += (base + e < N && taken[e] && !in_r0[e]) ? 1 : 0;
+  for (int e = 0; e < PER; ++e) cnt += (base + e < N && taken[e] && !in_r0[e]) ? 1 : 0;
+  group_sync(nt);
   int total;
   int pos = block_exclusive_scan(cnt, &total, nt, s);
 #pragma unroll
-  for (int e = 0; e < kPer; ++e)
+  for (int e = 0; e < PER; ++e)
     if (base + e < N && taken[e] && !in_r0[e] && pos < C) cand[static_cast<size_t>(b) * C + pos++] = base + e;
 }
 
@@ -255,18 +266,12 @@ __global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* __restrict_
 // Order key of a score with -0 and +0 equal (they tie, and the lower index wins).
 __device__ __forceinline__ uint32_t score_key(float v) { return float_order_key(v == 0.0f ? 0.0f : v); }
 
-struct TopkScratch {
-  unsigned int hist[256];
-  unsigned int wsum[32];
-  int digit, above;
-};
-
 __global__ void __launch_bounds__(kSelThreads)
     topk_replacement_kernel(const float* __restrict__ s_ref, const float* __restrict__ s_alt, int N, int K,
                             int32_t* __restrict__ inter, float* __restrict__ rho) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ TopkScratch s;
+  __shared__ RankScratch s;
   const int b = blockIdx.x, nt = blockDim.x, base = kPer * threadIdx.x;
   uint32_t key[kPer];
   bool in_ref[kPer], in_alt[kPer];
@@ -276,11 +281,12 @@ __global__ void __launch_bounds__(kSelThreads)
     in_ref[e] = false;
     in_alt[e] = false;
   }
-  block_take_top(key, in_ref, base, N, K, nt, s);
+  block_take_top<false>(key, in_ref, base, N, K, nt, s);
 #pragma unroll
   for (int e = 0; e < kPer; ++e)
     key[e] = base + e < N ? score_key(s_alt[static_cast<size_t>(b) * N + base + e]) : 0u;
-  block_take_top(key, in_alt, base, N, K, nt, s);
+  block_take_top<false>(key, in_alt, base, N, K, nt, s);
+  group_sync(nt);
   int c = 0;
 #pragma unroll
   for (int e = 0; e < kPer; ++e) c += (in_ref[e] && in_alt[e]) ? 1 : 0;
@@ -384,16 +390,25 @@ size_t select_workspace_layout(int B, int N, int d, int J, int R0, int C, bool g
   return off;
 }
 
+// Tokens per thread of a ranking block (at most 1024 threads) and its threads.
+template <class F>
+static cudaError_t with_per(int N, F f) {
+  const int per = (N + kSelThreads - 1) / kSelThreads, nt = ((N + per - 1) / per + 31) / 32 * 32;
+  switch (per) {
+    case 1: return f(std::integral_constant<int, 1>(), nt);
+    case 2: return f(std::integral_constant<int, 2>(), nt);
+    case 3: return f(std::integral_constant<int, 3>(), nt);
+    default: return f(std::integral_constant<int, 4>(), nt);
+  }
+}
+
 cudaError_t launch_select_stages12(const SelectPlan& p, const SelectWorkspace& ws, const float* A_cls, int32_t* idx,
                                    cudaStream_t stream) {
-  const int nt = ((p.N + kPer - 1) / kPer + 31) / 32 * 32;
-  auto args = [&](auto kern) {
-    return launch_pdl(kern, dim3(p.B), dim3(nt), 0, stream, ws.qdots, ws.q_pitch, ws.qnorm, ws.vnorm, A_cls, p.N,
-                      p.J, p.Kq, p.Ks, p.Kd, ws.kept12, ws.r0tok, idx);
-  };
-  if (nt <= 512) return args(select_stages12_kernel<512>);
-  if (nt <= 768) return args(select_stages12_kernel<768>);
-  return args(select_stages12_kernel<kSelThreads>);
+  return with_per(p.N, [&](auto per, int nt) {
+    constexpr int PER = decltype(per)::value;
+    return launch_pdl(select_stages12_kernel<PER>, dim3(p.B), dim3(nt), 0, stream, ws.qdots, ws.q_pitch, ws.qnorm,
+                      ws.vnorm, A_cls, p.N, p.J, p.Kq, p.Ks, p.Kd, ws.kept12, ws.r0tok, idx);
+  });
 }
 
 cudaError_t launch_query_dots(const SelectPlan& p, const SelectWorkspace& ws, cudaStream_t stream) {
@@ -448,6 +463,13 @@ cudaError_t launch_gram(const SelectPlan& p, const SelectWorkspace& ws, cudaStre
   g.D = ws.cdots;
   g.d_pitch = ws.cpitch;
   g.f32_out = true;
+  // few images: the narrowest tiles of which every CTA pair still takes one at
+  // most (one image of 576 tokens, whole selector call, us: 256 columns 56.0,
+  // 128 53.5, 64 52.4; three images, where 64 columns make a second round: 63.9,
+  // 60.9, 69.3)
+  const int pairs = num_sms() / 2, rows = p.B * ((p.N + 255) / 256);
+  for (int tn : {128, 64})
+    if (rows * ((p.N + tn - 1) / tn) <= pairs) g.tile_n = tn;
   return launch_gemm8(g, ws.vu, ws.vsum, ws.vu, ws.vsum, stream);
 }
 
@@ -464,13 +486,11 @@ cudaError_t launch_candidates(const SelectPlan& p, const SelectWorkspace& ws, cu
   const int C = ws.C;
   if (C <= 0) return cudaSuccess;
   const int R0 = p.Kq + p.Ks;
-  const int nt = ((p.N + kPer - 1) / kPer + 31) / 32 * 32;
-  auto go = [&](auto kern) {
-    return launch_pdl(kern, dim3(p.B), dim3(nt), 0, stream, ws.m, ws.r0_parts > 1 ? ws.mpart : nullptr,
-                      ws.r0_parts, ws.kept12, p.N, R0, C, ws.cand);
-  };
-  cudaError_t e = nt <= 512 ? go(select_candidates_kernel<512>)
-                            : (nt <= 768 ? go(select_candidates_kernel<768>) : go(select_candidates_kernel<kSelThreads>));
+  cudaError_t e = with_per(p.N, [&](auto per, int nt) {
+    constexpr int PER = decltype(per)::value;
+    return launch_pdl(select_candidates_kernel<PER>, dim3(p.B), dim3(nt), 0, stream, ws.m,
+                      ws.r0_parts > 1 ? ws.mpart : nullptr, ws.r0_parts, ws.kept12, p.N, R0, C, ws.cand);
+  });
   if (e != cudaSuccess) return e;
   const int rows = p.B * C;
   const int blocks = std::min((rows + 7) / 8, 4 * num_sms());

@@ -230,3 +230,19 @@ def test_select_from_two_host_threads_on_two_streams(p4q, dev):
         t.join()
     assert p4q.p4q_device_status() == 0
     assert not errors, errors
+
+
+@pytest.mark.parametrize("B,N,K,J", [(1, 576, 64, 3), (3, 576, 190, 5), (1, 1024, 300, 4), (1, 1025, 300, 4),
+                                     (2, 2049, 900, 3), (1, 3073, 500, 9), (2, 257, 257, 1), (5, 33, 7, 16)])
+def test_select_ranking_widths(p4q, dev, B, N, K, J):
+    """Token counts around one to four tokens per ranking thread, few images on
+    narrow token-pair tiles, and score rows whose ranked boundary lies in one
+    crowded bin (repeated saliency values, a few far outliers)."""
+    w = wl.Workload("t", B=B, N=N, d=256, K=K, T=0, J=J, seed=B * N + K, heavy_tail=False, linears=())
+    x = wl.selector_inputs(w)
+    A = np.floor(x.A * 4000).astype(np.float32) / 4000  # many ties, most of them in the lowest values
+    A[:, 0] = 1000.0
+    idx = p4q.select(torch.from_numpy(x.V).to(dev), torch.from_numpy(x.Q).to(dev), torch.from_numpy(A).to(dev), K)
+    torch.cuda.synchronize()
+    assert p4q.p4q_device_status() == 0
+    assert np.array_equal(idx.cpu().numpy(), oracle.select_batch(x.V, K, x.Q, A))
