@@ -57,16 +57,16 @@ struct DivScratch {
   RankScratch rank;
   int t, npool, tmin, nphase;
   unsigned long long tau;
-  __align__(16) unsigned long long skey[kPool];  // pool rounds: (m, slot) keys of the certain entries
+  __align__(16) uint32_t skey[kPool];   // pool rounds: order keys of the certain entries' m
+  int prank[kPool];                     // pool rounds: their ranks
   int sorted[kPool];                    // pool rounds: slots of the certain entries in key order
   int L;                                // pool rounds: length of the confirmed prefix
   int ptok[kPool];                      // pool slot -> token (ascending)
   float pm[kPool];                      // m of the pool tokens (bound, then exact)
-  unsigned int pmx[kPool];              // order key of the largest cosine to the pick columns
+  unsigned int pmx[kPool];              // order key of the largest cosine to the pick columns; pool rounds: of m
   int psum[kPool], pnorm[kPool];        // pool rows: sum of u, squared code norm
   float prs[kPool];                     // pool rows: rsqrtf of the squared code norm (0 for a zero row)
   int csum[kBrows], cnorm[kBrows];      // extra columns of the current chunk
-  float crs[kBrows];                    // their rsqrtf norms (candidate path)
   unsigned int keptbits[P4Q_MAX_TOKENS / 32];
   int16_t list[P4Q_MAX_TOKENS];         // the greedy picks, in order
   signed char slotof[P4Q_MAX_TOKENS];   // token -> pool slot, -1 outside the pool
@@ -81,76 +81,103 @@ struct DivScratch {
   __align__(16) float cp[kPool][kPool + 1]; // cos(ptok[i], ptok[j]) (Eq. 4, exact; padded: column writes)
 };
 
-// Greedy rounds on the pool, by the whole block (thread i < 128 owns pool
-// slot i), with exact m of the pool entries in s.pm. The next pick is the
-// smallest free (m, token) pair. A pool entry is certain to be in order while
-// its pair is at most tau (every token outside the pool is above tau and m
-// only grows). Per iteration the certain entries are ranked by their pairs
-// (each owner counts the smaller keys), giving c_0 < c_1 < ...; c_0 is the
-// next pick, and c_a the pick after c_0 .. c_{a-1} whenever none of their
-// cosines exceeds m(c_a) (nothing else can pass it: every other pair only
-// grows). The pairs (b < a) are checked in parallel; the longest such
-// prefix (at most kPickMax) is picked at once, the pool's m absorbs the
-// picks' cosines, and the picks are appended to s.list. Ends when Kd picks
-// are made or no entry is certain; s.t and s.pm hold the results.
+// Greedy rounds on the pool, by the whole block, with exact m of the pool
+// entries in s.pm. The next pick is the smallest free
+// (m, token) pair. A pool entry is certain to be in order while its pair is at
+// most tau (every token outside the pool is above tau and m only grows). Per
+// iteration the certain entries are ranked by their pairs (four warps per
+// 32 slots count the smaller keys, every load a broadcast), giving c_0 < c_1 < ...; c_0 is the next pick, and
+// c_a the pick after c_0 .. c_{a-1} whenever none of their cosines exceeds
+// m(c_a) (nothing else can pass it: every other pair only grows). The pairs
+// (b < a) are checked in parallel; the longest such prefix (at most kPickMax)
+// is picked at once, the pool's m absorbs the picks' cosines, and the picks
+// are appended to s.list. Ends when Kd picks are made or no entry is certain;
+// s.t and s.pm hold the results.
+// Two to five iterations make the picks of a 576-token image (about 30 each),
+// of about 3250 cycles (640 threads; 4000 with 768): half of it the 16 K key
+// comparisons of the ranks, bound by the integer pipe. With a thread per slot
+// in all but the pair check an iteration took 4300 (4700).
 template <int kThreads>
 __device__ void pool_rounds(int npool, int Kd, DivScratch& s) {
-  constexpr unsigned long long kNone = ~0ull;
-  const int tid = threadIdx.x;
+  constexpr uint32_t kNone = 0xFFFFFFFFu;
+  constexpr int kParts = 4;                    // warps per 32 slots
+  constexpr int kCheck = kThreads / kPickMax;  // threads per candidate of the pair check
+  static_assert(kPool == 128 && kPickMax == 64 && kThreads % 64 == 0 && kThreads >= kParts * kPool, "thread layout");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slot = tid & (kPool - 1), part = warp >> 2;  // (slot of the warp's lanes: 32 (warp % 4) + lane)
   const unsigned long long tau = s.tau;
-  bool alive = tid < npool;
+  if (tid < kPool) s.pmx[tid] = tid < npool ? float_order_key(s.pm[tid]) : kNone;
+  bool alive = tid < npool;  // of thread tid's slot, tid < kPool
   while (true) {
     const int t = s.t;  // every thread has passed the barrier that published it
     if (t >= Kd) break;
-    unsigned long long key = kNone;
-    if (alive) {
-      const unsigned long long pr = (static_cast<unsigned long long>(float_order_key(s.pm[tid])) << 32) | tid;
-      if (pr <= tau) key = pr;
+    bool certain = false;
+    if (tid < kPool) {
+      const uint32_t k = s.pmx[tid];
+      certain = alive && ((static_cast<unsigned long long>(k) << 32) | tid) <= tau;
+      s.skey[tid] = certain ? k : kNone;
+      s.prank[tid] = 0;
     }
-    if (tid < kPool) s.skey[tid] = key;
     if (tid == 0) s.L = kPickMax;
-    const int nc = __syncthreads_count(key != kNone);
+    const int nc = __syncthreads_count(certain);
     const int r = min(min(nc, Kd - t), kPickMax);
     if (r == 0) break;
-    // rank of each certain entry among them (keys are unique: the slot is in the low bits)
-    int rank = kPool;
-    if (key != kNone) {
-      rank = 0;
-#pragma unroll 8
-      for (int f = 0; f < kPool; f += 2) {
-        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(&s.skey[f]);
-        rank += (kk.x < key ? 1 : 0) + (kk.y < key ? 1 : 0);
+    // rank of each certain entry among them: the smaller keys, and the equal
+    // ones of lower slots (keys below kNone: no cosine's key is that large)
+    if (part < kParts) {
+      const uint32_t key = s.skey[slot];
+      int cnt = 0;
+      if (part != (warp & 3)) {
+        const uint32_t lim = key + (part < (warp & 3) ? 1u : 0u);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 k = *reinterpret_cast<const uint4*>(&s.skey[32 * part + 4 * i]);
+          cnt += (k.x < lim ? 1 : 0) + (k.y < lim ? 1 : 0) + (k.z < lim ? 1 : 0) + (k.w < lim ? 1 : 0);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 k = *reinterpret_cast<const uint4*>(&s.skey[32 * part + 4 * i]);
+          cnt += (k.x < key + (4 * i < lane ? 1u : 0u) ? 1 : 0) + (k.y < key + (4 * i + 1 < lane ? 1u : 0u) ? 1 : 0) +
+                 (k.z < key + (4 * i + 2 < lane ? 1u : 0u) ? 1 : 0) + (k.w < key + (4 * i + 3 < lane ? 1u : 0u) ? 1 : 0);
+        }
       }
-      if (rank < r) s.sorted[rank] = tid;
+      if (key != kNone) atomicAdd(&s.prank[slot], cnt);
     }
     __syncthreads();
+    const int rank = certain ? s.prank[tid] : kPool;
+    if (rank < r) s.sorted[rank] = tid;
+    __syncthreads();
     // pairs b < a < r: a violation (an earlier candidate raises c_a) ends the prefix at a
-    const int npairs = r * (r - 1) / 2;
-    for (int q = tid; q < npairs; q += kThreads) {
-      int a2 = static_cast<int>((1.0f + sqrtf(1.0f + 8.0f * static_cast<float>(q))) * 0.5f);
-      while (a2 * (a2 - 1) / 2 > q) --a2;
-      while ((a2 + 1) * a2 / 2 <= q) ++a2;
-      const int b2 = q - a2 * (a2 - 1) / 2;
-      const int ca = s.sorted[a2];
-      if (s.cp[s.sorted[b2]][ca] > s.pm[ca]) atomicMin(&s.L, a2);
+    {
+      const int a2 = tid & (kPickMax - 1);
+      bool bad = false;
+      if (a2 < r) {
+        const int ca = s.sorted[a2];
+        const float mc = s.pm[ca];
+#pragma unroll 4
+        for (int b2 = tid / kPickMax; b2 < a2; b2 += kCheck) bad |= s.cp[s.sorted[b2]][ca] > mc;
+      }
+      const unsigned int v = __ballot_sync(0xFFFFFFFFu, bad);
+      if (v != 0 && lane == __ffs(v) - 1) atomicMin(&s.L, a2);
     }
     __syncthreads();
     const int L = min(s.L, r);  // >= 1: c_0 never fails
-    if (alive) {
-      if (rank < L) {
-        alive = false;
-        const int tok = s.ptok[tid];
-        s.list[t + rank] = static_cast<int16_t>(tok);
-        atomicOr(&s.keptbits[tok >> 5], 1u << (tok & 31));
-      } else {
-        float m = s.pm[tid];
-#pragma unroll 8
-        for (int b2 = 0; b2 < L; ++b2) m = fmaxf(m, s.cp[s.sorted[b2]][tid]);
-        s.pm[tid] = m;
-      }
+    if (rank < L) {
+      alive = false;
+      const int tok = s.ptok[tid];
+      s.list[t + rank] = static_cast<int16_t>(tok);
+      atomicOr(&s.keptbits[tok >> 5], 1u << (tok & 31));
+    }
+    if (part < kParts) {
+      float mx = -INFINITY;
+#pragma unroll 4
+      for (int b2 = part; b2 < L; b2 += kParts) mx = fmaxf(mx, s.cp[s.sorted[b2]][slot]);
+      atomicMax(&s.pmx[slot], float_order_key(mx));
     }
     if (tid == 0) s.t = t + L;
     __syncthreads();
+    if (tid < kPool) s.pm[tid] = order_key_float(s.pmx[tid]);
   }
 }
 
@@ -169,7 +196,8 @@ struct DivArgs {
   int32_t* idx;            // [B, K]
 };
 
-template <int kThreads>
+// Token i of the image is held by thread i / PER (element i % PER).
+template <int kThreads, int PER>
 __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -177,9 +205,9 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   constexpr int kWarps = kThreads / 32;
   const int b = blockIdx.x, N = a.N, d = a.d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tpg = ((N + kPer - 1) / kPer + 31) / 32 * 32;  // token owners (group 0)
+  const int tpg = ((N + PER - 1) / PER + 31) / 32 * 32;  // token owners (group 0)
   const bool g0 = threadIdx.x < tpg;
-  const int base = kPer * threadIdx.x;
+  const int base = PER * threadIdx.x;
   const int words = (N + 31) / 32;
   const size_t row0 = static_cast<size_t>(b) * N;
 
@@ -201,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   }
   for (int i = threadIdx.x; i < N; i += kThreads) {
     s.slotof[i] = -1;
-    s.candof[i] = -1;
+    s.candof[i] = a.cand ? -1 : static_cast<int16_t>(i);  // (without candidates, C = N: the token itself)
   }
   tc_fence_before();
   __syncthreads();
@@ -211,27 +239,25 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   pdl_wait();  // R0 bits and maxima come from the kernels before
   pdl_launch_dependents();
   for (int w = threadIdx.x; w < words; w += kThreads) s.keptbits[w] = a.kept12[static_cast<size_t>(b) * words + w];
-  __syncthreads();  // candof is cleared
-  for (int c = threadIdx.x; c < a.C; c += kThreads)
-    s.candof[a.cand ? a.cand[static_cast<size_t>(b) * a.C + c] : c] = static_cast<int16_t>(c);
-  __syncthreads();
+  if (a.cand)
+    for (int c = threadIdx.x; c < a.C; c += kThreads)
+      s.candof[a.cand[static_cast<size_t>(b) * a.C + c]] = static_cast<int16_t>(c);
 
-  bool kept[kPer];
-  float m[kPer];
-  int ex[kPer];  // m of the token is exact up to the first ex picks
+  bool kept[PER];
+  float m[PER];
+  int ex[PER];  // m of the token is exact up to the first ex picks
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) {
+  for (int e = 0; e < PER; ++e) {
     const int i = base + e;
-    kept[e] = g0 && i < N && ((s.keptbits[i >> 5] >> (i & 31)) & 1u);
-    m[e] = -INFINITY;
+    kept[e] = false;  // (set from the bits at the top of each phase)
+    m[e] = g0 && i < N && a.R0 > 0 ? a.m[row0 + i] : -INFINITY;
     ex[e] = 0;
-    if (g0 && i < N && !kept[e] && a.R0 > 0) m[e] = a.m[row0 + i];
   }
   const int KB = d / kBK;
   const int phase_limit = a.Kd * (N / kPool + 2) + 8;
   int g = 0;       // k-blocks staged so far (mbarrier phases of bar_full / bar_empty)
   int chunks = 0;  // accumulators completed so far (phases of bar_acc)
-  uint32_t key[kPer];
+  uint32_t key[PER];
 
   while (true) {
     __syncthreads();
@@ -242,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
       atomicOr(&g_diverse_err, kErrTimeout);
     }
 #pragma unroll
-    for (int e = 0; e < kPer; ++e)
+    for (int e = 0; e < PER; ++e)
       if (g0 && base + e < N && ((s.keptbits[(base + e) >> 5] >> ((base + e) & 31)) & 1u)) kept[e] = true;
     // ---- 1. pool: the q smallest free (bound, token) pairs, in token order
     const int nfree = N - a.R0 - t;
@@ -250,16 +276,16 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     if (threadIdx.x == 0) s.tmin = t;
     int npool = 0;
     if (g0) {
-      bool member[kPer];
+      bool member[PER];
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) {
+      for (int e = 0; e < PER; ++e) {
         member[e] = kept[e];
         key[e] = (base + e < N) ? ~float_order_key(m[e]) : 0u;
       }
       block_take_top<true>(key, member, base, N, q, tpg, s.rank);
       int cnt = 0, emin = t;
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) {
+      for (int e = 0; e < PER; ++e) {
         const bool in = base + e < N && member[e] && !kept[e];
         cnt += in ? 1 : 0;
         emin = in ? min(emin, ex[e]) : emin;
@@ -267,17 +293,13 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
       group_sync(tpg);
       int pos = block_exclusive_scan(cnt, &npool, tpg, s.rank);
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) {
+      for (int e = 0; e < PER; ++e) {
         if (base + e < N && member[e] && !kept[e]) {
           const int i = base + e;
           s.ptok[pos] = i;
           s.pm[pos] = m[e];
           s.pmx[pos] = 0u;  // below the key of every float
-          s.psum[pos] = a.vsum[row0 + i];
-          s.pnorm[pos] = a.vnorm[row0 + i];
-          s.prs[pos] = s.pnorm[pos] > 0 ? rsqrtf(static_cast<float>(s.pnorm[pos])) : 0.0f;
           s.slotof[i] = static_cast<signed char>(pos);
-          s.pci[pos] = s.candof[i];
           ++pos;
         }
       }
@@ -289,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     const int tmin = s.tmin;
     const int ncp = t - tmin;  // picks whose cosines some pool bound has not seen
     // tau: the largest pool pair (everything certain when the pool holds every free token)
-    if (warp == 0) {
+    if (warp == kWarps - 1) {
       unsigned long long mx = 0;
 #pragma unroll
       for (int k = 0; k < kPoolPer; ++k) {
@@ -310,73 +332,115 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     bool mine_ok = true;
     for (int r = threadIdx.x; r < npool + ncp; r += kThreads) {
       const int tok = r < npool ? s.ptok[r] : s.list[tmin + r - npool];
-      mine_ok = mine_ok && s.candof[tok] >= 0;
+      const int ci = s.candof[tok];
+      mine_ok = mine_ok && ci >= 0;
+      if (r < npool) {  // its row's data (a thread per slot: one global latency)
+        const int ns = a.vnorm[row0 + tok];
+        s.psum[r] = a.vsum[row0 + tok];
+        s.pnorm[r] = ns;
+        s.prs[r] = ns > 0 ? rsqrtf(static_cast<float>(ns)) : 0.0f;
+        s.pci[r] = ci;
+      }
     }
     const bool from_cand = __syncthreads_and(mine_ok) != 0;
     if (from_cand) {
       const float* cd = a.cdots + static_cast<size_t>(b) * a.C * a.cpitch;
-      // the pool block, one warp per row, four columns per lane in flight
-      for (int e = warp; e < npool; e += kWarps) {
-        const float* row = cd + static_cast<size_t>(s.pci[e]) * a.cpitch;
-        float v[kPoolPer];
+      const int32_t* cn = a.candnorm + static_cast<size_t>(b) * a.C;
+      // the unseen picks' columns (in the stage ring, which nothing uses here)
+      int* pick_c = reinterpret_cast<int*>(stages);
+      int* pick_n = pick_c + P4Q_MAX_TOKENS;
+      float* pick_rs = reinterpret_cast<float*>(pick_n + P4Q_MAX_TOKENS);
+      static_assert(P4Q_MAX_TOKENS * 12 <= kStages * kStageBytes, "pick columns");
+      for (int c = threadIdx.x; c < ncp; c += kThreads) {
+        const int cj = s.candof[s.list[tmin + c]];
+        const int nj = cn[cj];
+        pick_c[c] = cj;
+        pick_n[c] = nj;
+        pick_rs[c] = nj > 0 ? rsqrtf(static_cast<float>(nj)) : 0.0f;
+      }
+      // the pool block, a warp per row, four rows of four columns per lane in
+      // flight; it is symmetric: each pair once (f >= e), written both ways
+      constexpr int kR = 4;
+      int fc[kPoolPer], fn[kPoolPer];
 #pragma unroll
-        for (int k = 0; k < kPoolPer; ++k) {
-          const int f = lane + 32 * k;
-          v[k] = f < npool ? __ldg(row + s.pci[f]) : 0.0f;
+      for (int k = 0; k < kPoolPer; ++k) {
+        const int f = lane + 32 * k;
+        fc[k] = f < npool ? s.pci[f] : 0;
+        fn[k] = f < npool ? s.pnorm[f] : 0;
+      }
+      for (int e0 = warp; e0 < npool; e0 += kR * kWarps) {
+        float v[kR][kPoolPer];
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+          const int e = e0 + j * kWarps;
+          const float* row = cd + static_cast<size_t>(e < npool ? s.pci[e] : 0) * a.cpitch;
+#pragma unroll
+          for (int k = 0; k < kPoolPer; ++k) {
+            const int f = lane + 32 * k;
+            v[j][k] = f < npool && f >= e ? __ldg(row + fc[k]) : 0.0f;
+          }
         }
-        const int ne = s.pnorm[e];
-        // the block is symmetric: each pair once (f >= e), written both ways
 #pragma unroll
-        for (int k = 0; k < kPoolPer; ++k) {
-          const int f = lane + 32 * k;
-          if (f < npool && f >= e) {
-            const float c = code_cosine(static_cast<int>(v[k]), ne, s.pnorm[f]);
-            s.cp[e][f] = c;
-            s.cp[f][e] = c;
+        for (int j = 0; j < kR; ++j) {
+          const int e = e0 + j * kWarps;
+#pragma unroll
+          for (int k = 0; k < kPoolPer; ++k) {
+            const int f = lane + 32 * k;
+            if (f < npool && f >= e) {
+              const float c = code_cosine(static_cast<int>(v[j][k]), s.pnorm[e], fn[k]);
+              s.cp[e][f] = c;
+              s.cp[f][e] = c;
+            }
           }
         }
       }
-      // per pool row: the largest cosine to the unseen picks (chunks of 128
-      // picks with their candidate index and norms in shared memory),
-      // approximate first, then exact for the columns near it
-      const int32_t* cn = a.candnorm + static_cast<size_t>(b) * a.C;
-      for (int c0 = 0; c0 < ncp; c0 += kBrows) {
-        const int nc2 = min(kBrows, ncp - c0);
-        __syncthreads();  // the previous chunk's column data is no longer read
-        for (int c = threadIdx.x; c < nc2; c += kThreads) {
-          const int cj = s.candof[s.list[tmin + c0 + c]];
-          const int nj = cn[cj];
-          s.csum[c] = cj;  // candidate index of the column
-          s.cnorm[c] = nj;
-          s.crs[c] = nj > 0 ? rsqrtf(static_cast<float>(nj)) : 0.0f;
-        }
+      // per pool row: the largest cosine to the unseen picks, 128 columns of
+      // four rows at a time: approximate, then exact for the columns near the
+      // largest so far (from the row's bound on: less does not raise it)
+      if (ncp > 0) {
         __syncthreads();
-        for (int e = warp; e < npool; e += kWarps) {
-          const float* row = cd + static_cast<size_t>(s.pci[e]) * a.cpitch;
-          float v[kBrows / 32];
+        for (int e0 = warp; e0 < npool; e0 += kR * kWarps) {
+          float amax[kR], emax[kR], rs[kR];
+          const float* row[kR];
 #pragma unroll
-          for (int k = 0; k < kBrows / 32; ++k) {
-            const int c = lane + 32 * k;
-            v[k] = c < nc2 ? __ldg(row + s.csum[c]) : 0.0f;
+          for (int j = 0; j < kR; ++j) {
+            const int e = min(e0 + j * kWarps, npool - 1);
+            amax[j] = s.pm[e];
+            emax[j] = -INFINITY;
+            rs[j] = s.prs[e];
+            row[j] = cd + static_cast<size_t>(s.pci[e]) * a.cpitch;
           }
-          float amax = -INFINITY;
+          for (int c0 = 0; c0 < ncp; c0 += 128) {
+            float v[kR][4];
 #pragma unroll
-          for (int k = 0; k < kBrows / 32; ++k) {
-            const int c = lane + 32 * k;
-            if (c < nc2) amax = fmaxf(amax, v[k] * s.prs[e] * s.crs[c]);
+            for (int k = 0; k < 4; ++k) {
+              const int c = c0 + lane + 32 * k;
+              const int cj = pick_c[min(c, ncp - 1)];
+#pragma unroll
+              for (int j = 0; j < kR; ++j) v[j][k] = __ldg(row[j] + cj);
+            }
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+              float ap[4], am = amax[j];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                ap[k] = v[j][k] * rs[j] * pick_rs[min(c0 + lane + 32 * k, ncp - 1)];
+                am = fmaxf(am, ap[k]);
+              }
+              amax[j] = order_key_float(__reduce_max_sync(0xFFFFFFFFu, float_order_key(am)));
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                if (ap[k] >= amax[j] - kCosMargin)
+                  emax[j] = fmaxf(emax[j], code_cosine(static_cast<int>(v[j][k]),
+                                                       s.pnorm[min(e0 + j * kWarps, npool - 1)],
+                                                       pick_n[min(c0 + lane + 32 * k, ncp - 1)]));
+            }
           }
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
-          float emax = -INFINITY;
-#pragma unroll
-          for (int k = 0; k < kBrows / 32; ++k) {
-            const int c = lane + 32 * k;
-            if (c < nc2 && v[k] * s.prs[e] * s.crs[c] >= amax - kCosMargin)
-              emax = fmaxf(emax, code_cosine(static_cast<int>(v[k]), s.pnorm[e], s.cnorm[c]));
+          for (int j = 0; j < kR; ++j) {
+            const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, float_order_key(emax[j]));
+            if (lane == 0 && e0 + j * kWarps < npool) s.pmx[e0 + j * kWarps] = mx;
           }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) emax = fmaxf(emax, __shfl_xor_sync(0xFFFFFFFFu, emax, o));
-          if (lane == 0) s.pmx[e] = max(s.pmx[e], float_order_key(emax));
         }
       }
       __syncthreads();
@@ -527,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     const int tn = s.t;
     if (g0) {
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) {
+      for (int e = 0; e < PER; ++e) {
         const int i = base + e;
         if (i < N && s.slotof[i] >= 0) {
           const int slot = s.slotof[i];
@@ -546,12 +610,12 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   if (g0) {
     int cnt = 0;
 #pragma unroll
-    for (int e = 0; e < kPer; ++e)
+    for (int e = 0; e < PER; ++e)
       cnt += (base + e < N && ((s.keptbits[(base + e) >> 5] >> ((base + e) & 31)) & 1u)) ? 1 : 0;
     int total;
     int pos = block_exclusive_scan(cnt, &total, tpg, s.rank);
 #pragma unroll
-    for (int e = 0; e < kPer; ++e)
+    for (int e = 0; e < PER; ++e)
       if (base + e < N && ((s.keptbits[(base + e) >> 5] >> ((base + e) & 31)) & 1u) && pos < a.K)
         a.idx[static_cast<size_t>(b) * a.K + pos++] = base + e;
   }
@@ -594,17 +658,22 @@ cudaError_t launch_select_diverse(const SelectPlan& p, const SelectWorkspace& ws
   a.K = p.K;
   a.Kd = p.Kd;
   a.idx = idx;
-  const int tpg = ((p.N + kPer - 1) / kPer + 31) / 32 * 32;
   auto go = [&](auto kern, int threads) -> cudaError_t {
-    static bool attr_set = false;  // one flag per instantiation
-    (void)attr_set;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDivSmem));
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(p.B), dim3(threads), kDivSmem, stream, a);
   };
-  if (tpg <= 512) return go(select_diverse_kernel<512>, 512);
-  if (tpg <= 768) return go(select_diverse_kernel<768>, 768);
-  return go(select_diverse_kernel<1024>, 1024);
+  // a token per thread where a block allows (the ranking of the pool and the
+  // scatter around it, cycles per phase: 576 tokens on 144 threads of four each
+  // 10.0 k, one each 6.4 k), and the narrowest of these blocks: barriers cost
+  // by the warp. Past 768 tokens two or four each (three: more registers than
+  // 1024 threads leave).
+  if (p.N <= 512) return go(select_diverse_kernel<512, 1>, 512);
+  if (p.N <= 640) return go(select_diverse_kernel<640, 1>, 640);
+  if (p.N <= 768) return go(select_diverse_kernel<768, 1>, 768);
+  if (p.N <= 1536) return go(select_diverse_kernel<768, 2>, 768);
+  if (p.N <= 3072) return go(select_diverse_kernel<768, 4>, 768);
+  return go(select_diverse_kernel<1024, 4>, 1024);
 }
 
 unsigned int diverse_read_and_clear_error() {

@@ -107,6 +107,9 @@ __device__ __forceinline__ void find_digit(int need, Scratch& s) {
 // lies in, a second one splits that bin; when the bin holds at most 32 tokens
 // (it nearly always does after one or two: scores spread over the range), one
 // warp ranks those and publishes the last pair taken: five or seven barriers.
+// The counts are plain shared atomics: combining a warp's equal bins by
+// match_any first costs more than the collisions that it saves (whole selector
+// call, 8 images of 2880 heavy-tailed tokens: 229 us with it, 214 without).
 // Otherwise (many equal scores, non-finite values) the bin's tokens go through
 // a radix select of their keys, 8 bits per pass, as every ranking did before
 // (about 20 barriers).
@@ -158,9 +161,7 @@ __device__ void block_take_top(const uint32_t (&key)[PER], bool (&kept)[PER], in
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
       bin[e] = static_cast<int>(x[e]);
-      // (aggregated per warp: a heavy-tailed score has most tokens in one bin)
-      const unsigned peers = __match_any_sync(0xFFFFFFFFu, live[e] ? bin[e] : 256);
-      if (live[e] && (__ffs(peers) - 1) == lane) atomicAdd(&s.hist[bin[e]], static_cast<unsigned>(__popc(peers)));
+      if (live[e]) atomicAdd(&s.hist[bin[e]], 1u);
     }
     group_sync(nt);
     if (warp == 0) find_digit(need, s);

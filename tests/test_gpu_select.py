@@ -246,3 +246,16 @@ def test_select_ranking_widths(p4q, dev, B, N, K, J):
     torch.cuda.synchronize()
     assert p4q.p4q_device_status() == 0
     assert np.array_equal(idx.cpu().numpy(), oracle.select_batch(x.V, K, x.Q, A))
+
+
+@pytest.mark.parametrize("N,K", [(512, 300), (513, 200), (640, 480), (641, 129), (768, 400), (769, 300), (1536, 700),
+                                 (1537, 260), (3072, 900), (3073, 400), (4096, 1000)])
+def test_diversity_block_widths(p4q, dev, N, K):
+    """Stage 3 at the edges of its block widths and of one, two and four tokens
+    per thread; many picks (several per iteration, several pools)."""
+    w = wl.Workload("t", B=2, N=N, d=256, K=K, T=0, J=2, seed=N + K, heavy_tail=False, linears=())
+    x = wl.selector_inputs(w)
+    idx = p4q.select(torch.from_numpy(x.V).to(dev), torch.from_numpy(x.Q).to(dev), torch.from_numpy(x.A).to(dev), K)
+    torch.cuda.synchronize()
+    assert p4q.p4q_device_status() == 0
+    assert np.array_equal(idx.cpu().numpy(), oracle.select_batch(x.V, K, x.Q, x.A))
