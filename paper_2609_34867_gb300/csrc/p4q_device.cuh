@@ -417,6 +417,12 @@ __device__ __forceinline__ uint32_t float_order_key(float f) {
 // ---------------------------------------------------------------- clusters / CTA pairs
 namespace p4q {
 
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));

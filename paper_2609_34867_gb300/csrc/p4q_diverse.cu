@@ -4,7 +4,8 @@
 // is empty); each of the K_d rounds keeps the free token with the smallest
 // m (lower index on ties) and m absorbs its cosines.
 //
-// One CTA per image. The largest cosine of every token to R0 comes from the
+// One CTA per image (and, up to 32 images, three helpers that share phase 2's
+// cosines). The largest cosine of every token to R0 comes from the
 // tensor-core GEMM before this kernel (its cosine-max epilogue, or a row pass
 // over its int32 tiles; in Gram mode a row pass over the token-pair GEMM)
 // as m. After that no cosine row of the whole image is ever formed. The kernel holds, for every free token, a
@@ -78,8 +79,11 @@ struct DivScratch {
   uint64_t bar_done;                    // MMA commit at teardown -> nothing in flight
   uint32_t tmem_slot;
   volatile int abort_flag;
-  __align__(16) float cp[kPool][kPool + 1]; // cos(ptok[i], ptok[j]) (Eq. 4, exact; padded: column writes)
+  int go, ncp;                          // to the helper CTAs: another phase's cosines, and its unseen picks
+  __align__(16) float cp[kPool][kPool + 1]; // cos(ptok[i], ptok[j]), i <= j (Eq. 4, exact; padded: column reads)
 };
+
+__device__ __forceinline__ float pool_cos(const DivScratch& s, int i, int j) { return s.cp[min(i, j)][max(i, j)]; }
 
 // Greedy rounds on the pool, by the whole block, with exact m of the pool
 // entries in s.pm. The next pick is the smallest free
@@ -156,7 +160,7 @@ __device__ void pool_rounds(int npool, int Kd, DivScratch& s) {
         const int ca = s.sorted[a2];
         const float mc = s.pm[ca];
 #pragma unroll 4
-        for (int b2 = tid / kPickMax; b2 < a2; b2 += kCheck) bad |= s.cp[s.sorted[b2]][ca] > mc;
+        for (int b2 = tid / kPickMax; b2 < a2; b2 += kCheck) bad |= pool_cos(s, s.sorted[b2], ca) > mc;
       }
       const unsigned int v = __ballot_sync(0xFFFFFFFFu, bad);
       if (v != 0 && lane == __ffs(v) - 1) atomicMin(&s.L, a2);
@@ -172,7 +176,7 @@ __device__ void pool_rounds(int npool, int Kd, DivScratch& s) {
     if (part < kParts) {
       float mx = -INFINITY;
 #pragma unroll 4
-      for (int b2 = part; b2 < L; b2 += kParts) mx = fmaxf(mx, s.cp[s.sorted[b2]][slot]);
+      for (int b2 = part; b2 < L; b2 += kParts) mx = fmaxf(mx, pool_cos(s, s.sorted[b2], slot));
       atomicMax(&s.pmx[slot], float_order_key(mx));
     }
     if (tid == 0) s.t = t + L;
@@ -196,6 +200,150 @@ struct DivArgs {
   int32_t* idx;            // [B, K]
 };
 
+struct PickCols {
+  int* c;     // candidate index
+  int* n;     // squared code norm
+  float* rs;  // its rsqrtf (0 for a zero row)
+};
+
+__device__ __forceinline__ PickCols pick_cols(uint8_t* stages) {
+  static_assert(P4Q_MAX_TOKENS * 12 <= kStages * kStageBytes, "pick columns");
+  int* c = reinterpret_cast<int*>(stages);
+  return PickCols{c, c + P4Q_MAX_TOKENS, reinterpret_cast<float*>(c + 2 * P4Q_MAX_TOKENS)};
+}
+
+// The same variable of CTA rank of the cluster (a generic address).
+template <class T>
+__device__ __forceinline__ T* cluster_ptr(T* p, uint32_t rank) {
+  uint64_t r;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+  return reinterpret_cast<T*>(r);
+}
+
+// Pool rows rank, rank + cs, ... of a phase whose tokens are all candidates:
+// their exact cosines to the pool (into out.cp) and the largest to the ncp
+// unseen picks pk (into out.pmx), from the candidates' dot products; the
+// pool's data from s.
+template <int kThreads>
+__device__ __forceinline__ void cand_cosines(const DivArgs& a, int b, int npool, int ncp, int rank, int cs,
+                                             const DivScratch& s, const PickCols& pk, DivScratch& out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int step = cs * (kThreads / 32);
+  const float* cd = a.cdots + static_cast<size_t>(b) * a.C * a.cpitch;
+  // the pool block, a warp per row, two rows of four columns per lane in
+  // flight; it is symmetric: each pair once (f >= e)
+  constexpr int kR = 2;
+  int fc[kPoolPer], fn[kPoolPer];
+#pragma unroll
+  for (int k = 0; k < kPoolPer; ++k) {
+    const int f = lane + 32 * k;
+    fc[k] = f < npool ? s.pci[f] : 0;
+    fn[k] = f < npool ? s.pnorm[f] : 0;
+  }
+  for (int e0 = rank + cs * warp; e0 < npool; e0 += kR * step) {
+    float v[kR][kPoolPer];
+#pragma unroll
+    for (int j = 0; j < kR; ++j) {
+      const int e = e0 + j * step;
+      const float* row = cd + static_cast<size_t>(e < npool ? s.pci[e] : 0) * a.cpitch;
+#pragma unroll
+      for (int k = 0; k < kPoolPer; ++k) {
+        const int f = lane + 32 * k;
+        v[j][k] = f < npool && f >= e ? __ldg(row + fc[k]) : 0.0f;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kR; ++j) {
+      const int e = e0 + j * step;
+#pragma unroll
+      for (int k = 0; k < kPoolPer; ++k) {
+        const int f = lane + 32 * k;
+        if (f < npool && f >= e) {
+          const float c = code_cosine(static_cast<int>(v[j][k]), s.pnorm[e], fn[k]);
+          out.cp[e][f] = c;
+        }
+      }
+    }
+  }
+  // per pool row: the largest cosine to the unseen picks, 128 columns of
+  // two rows at a time: approximate, then exact for the columns near the
+  // largest so far (from the row's bound on: less does not raise it)
+  if (ncp > 0) {
+    for (int e0 = rank + cs * warp; e0 < npool; e0 += kR * step) {
+      float amax[kR], emax[kR], rs[kR];
+      const float* row[kR];
+#pragma unroll
+      for (int j = 0; j < kR; ++j) {
+        const int e = min(e0 + j * step, npool - 1);
+        amax[j] = s.pm[e];
+        emax[j] = -INFINITY;
+        rs[j] = s.prs[e];
+        row[j] = cd + static_cast<size_t>(s.pci[e]) * a.cpitch;
+      }
+      for (int c0 = 0; c0 < ncp; c0 += 128) {
+        float v[kR][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int cj = pk.c[min(c0 + lane + 32 * k, ncp - 1)];
+#pragma unroll
+          for (int j = 0; j < kR; ++j)
+            if (e0 + j * step < npool) v[j][k] = __ldg(row[j] + cj);
+        }
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+          if (e0 + j * step >= npool) break;
+          float ap[4], am = amax[j];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            ap[k] = v[j][k] * rs[j] * pk.rs[min(c0 + lane + 32 * k, ncp - 1)];
+            am = fmaxf(am, ap[k]);
+          }
+          amax[j] = order_key_float(__reduce_max_sync(0xFFFFFFFFu, float_order_key(am)));
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (ap[k] >= amax[j] - kCosMargin)
+              emax[j] = fmaxf(emax[j], code_cosine(static_cast<int>(v[j][k]),
+                                                   s.pnorm[min(e0 + j * step, npool - 1)],
+                                                   pk.n[min(c0 + lane + 32 * k, ncp - 1)]));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kR; ++j) {
+        const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, float_order_key(emax[j]));
+        if (lane == 0 && e0 + j * step < npool) out.pmx[e0 + j * step] = mx;
+      }
+    }
+  }
+}
+
+// A helper CTA: its share of the cosines of each phase that takes them from
+// the candidates' dot products, written into the first CTA's shared memory.
+template <int kThreads>
+__device__ void diverse_helper(const DivArgs& a, int b, int rank, int cs, DivScratch& s, uint8_t* stages) {
+  DivScratch& s0 = *cluster_ptr(&s, 0);
+  const PickCols pk = pick_cols(stages), pk0 = pick_cols(cluster_ptr(stages, 0));
+  while (true) {
+    cluster_sync();  // the phase's pool and picks are in place, or the picks are complete
+    if (!s0.go) break;
+    const int npool = s0.npool, ncp = s0.ncp;
+    for (int r = threadIdx.x; r < npool; r += kThreads) {
+      s.pci[r] = s0.pci[r];
+      s.pnorm[r] = s0.pnorm[r];
+      s.prs[r] = s0.prs[r];
+      s.pm[r] = s0.pm[r];
+    }
+    for (int c = threadIdx.x; c < ncp; c += kThreads) {
+      pk.c[c] = pk0.c[c];
+      pk.n[c] = pk0.n[c];
+      pk.rs[c] = pk0.rs[c];
+    }
+    __syncthreads();
+    cand_cosines<kThreads>(a, b, npool, ncp, rank, cs, s, pk, s0);
+    cluster_sync();
+  }
+  cluster_sync();  // the first CTA stays until every helper has read its word
+}
+
 // Token i of the image is held by thread i / PER (element i % PER).
 template <int kThreads, int PER>
 __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivArgs a) {
@@ -203,7 +351,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   DivScratch& s = *reinterpret_cast<DivScratch*>(stages + kStages * kStageBytes);
   constexpr int kWarps = kThreads / 32;
-  const int b = blockIdx.x, N = a.N, d = a.d;
+  const int cs = static_cast<int>(cluster_nctarank()), rank = static_cast<int>(cluster_ctarank());
+  const int b = blockIdx.x / cs, N = a.N, d = a.d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tpg = ((N + PER - 1) / PER + 31) / 32 * 32;  // token owners (group 0)
   const bool g0 = threadIdx.x < tpg;
@@ -211,6 +360,12 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   const int words = (N + 31) / 32;
   const size_t row0 = static_cast<size_t>(b) * N;
 
+  if (rank > 0) {
+    pdl_wait();
+    pdl_launch_dependents();
+    diverse_helper<kThreads>(a, b, rank, cs, s, stages);
+    return;
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s.bar_full[i], kThreads / 32 - 1);
@@ -344,106 +499,25 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     }
     const bool from_cand = __syncthreads_and(mine_ok) != 0;
     if (from_cand) {
-      const float* cd = a.cdots + static_cast<size_t>(b) * a.C * a.cpitch;
-      const int32_t* cn = a.candnorm + static_cast<size_t>(b) * a.C;
       // the unseen picks' columns (in the stage ring, which nothing uses here)
-      int* pick_c = reinterpret_cast<int*>(stages);
-      int* pick_n = pick_c + P4Q_MAX_TOKENS;
-      float* pick_rs = reinterpret_cast<float*>(pick_n + P4Q_MAX_TOKENS);
-      static_assert(P4Q_MAX_TOKENS * 12 <= kStages * kStageBytes, "pick columns");
+      const PickCols pk = pick_cols(stages);
+      const int32_t* cn = a.candnorm + static_cast<size_t>(b) * a.C;
       for (int c = threadIdx.x; c < ncp; c += kThreads) {
         const int cj = s.candof[s.list[tmin + c]];
         const int nj = cn[cj];
-        pick_c[c] = cj;
-        pick_n[c] = nj;
-        pick_rs[c] = nj > 0 ? rsqrtf(static_cast<float>(nj)) : 0.0f;
+        pk.c[c] = cj;
+        pk.n[c] = nj;
+        pk.rs[c] = nj > 0 ? rsqrtf(static_cast<float>(nj)) : 0.0f;
       }
-      // the pool block, a warp per row, four rows of four columns per lane in
-      // flight; it is symmetric: each pair once (f >= e), written both ways
-      constexpr int kR = 4;
-      int fc[kPoolPer], fn[kPoolPer];
-#pragma unroll
-      for (int k = 0; k < kPoolPer; ++k) {
-        const int f = lane + 32 * k;
-        fc[k] = f < npool ? s.pci[f] : 0;
-        fn[k] = f < npool ? s.pnorm[f] : 0;
+      if (threadIdx.x == 0) {
+        s.go = 1;
+        s.ncp = ncp;
       }
-      for (int e0 = warp; e0 < npool; e0 += kR * kWarps) {
-        float v[kR][kPoolPer];
-#pragma unroll
-        for (int j = 0; j < kR; ++j) {
-          const int e = e0 + j * kWarps;
-          const float* row = cd + static_cast<size_t>(e < npool ? s.pci[e] : 0) * a.cpitch;
-#pragma unroll
-          for (int k = 0; k < kPoolPer; ++k) {
-            const int f = lane + 32 * k;
-            v[j][k] = f < npool && f >= e ? __ldg(row + fc[k]) : 0.0f;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < kR; ++j) {
-          const int e = e0 + j * kWarps;
-#pragma unroll
-          for (int k = 0; k < kPoolPer; ++k) {
-            const int f = lane + 32 * k;
-            if (f < npool && f >= e) {
-              const float c = code_cosine(static_cast<int>(v[j][k]), s.pnorm[e], fn[k]);
-              s.cp[e][f] = c;
-              s.cp[f][e] = c;
-            }
-          }
-        }
-      }
-      // per pool row: the largest cosine to the unseen picks, 128 columns of
-      // four rows at a time: approximate, then exact for the columns near the
-      // largest so far (from the row's bound on: less does not raise it)
-      if (ncp > 0) {
-        __syncthreads();
-        for (int e0 = warp; e0 < npool; e0 += kR * kWarps) {
-          float amax[kR], emax[kR], rs[kR];
-          const float* row[kR];
-#pragma unroll
-          for (int j = 0; j < kR; ++j) {
-            const int e = min(e0 + j * kWarps, npool - 1);
-            amax[j] = s.pm[e];
-            emax[j] = -INFINITY;
-            rs[j] = s.prs[e];
-            row[j] = cd + static_cast<size_t>(s.pci[e]) * a.cpitch;
-          }
-          for (int c0 = 0; c0 < ncp; c0 += 128) {
-            float v[kR][4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int c = c0 + lane + 32 * k;
-              const int cj = pick_c[min(c, ncp - 1)];
-#pragma unroll
-              for (int j = 0; j < kR; ++j) v[j][k] = __ldg(row[j] + cj);
-            }
-#pragma unroll
-            for (int j = 0; j < kR; ++j) {
-              float ap[4], am = amax[j];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                ap[k] = v[j][k] * rs[j] * pick_rs[min(c0 + lane + 32 * k, ncp - 1)];
-                am = fmaxf(am, ap[k]);
-              }
-              amax[j] = order_key_float(__reduce_max_sync(0xFFFFFFFFu, float_order_key(am)));
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                if (ap[k] >= amax[j] - kCosMargin)
-                  emax[j] = fmaxf(emax[j], code_cosine(static_cast<int>(v[j][k]),
-                                                       s.pnorm[min(e0 + j * kWarps, npool - 1)],
-                                                       pick_n[min(c0 + lane + 32 * k, ncp - 1)]));
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < kR; ++j) {
-            const uint32_t mx = __reduce_max_sync(0xFFFFFFFFu, float_order_key(emax[j]));
-            if (lane == 0 && e0 + j * kWarps < npool) s.pmx[e0 + j * kWarps] = mx;
-          }
-        }
-      }
-      __syncthreads();
+      if (cs > 1) cluster_sync();
+      else __syncthreads();
+      cand_cosines<kThreads>(a, b, npool, ncp, 0, cs, s, pk, s);
+      if (cs > 1) cluster_sync();
+      else __syncthreads();
     } else {
     // the rows this phase reads, toward L2 ahead of the staged loads
     for (int r = threadIdx.x; r < npool + ncp; r += kThreads) {
@@ -606,6 +680,11 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
       }
     }
   }
+  if (cs > 1) {  // the helpers leave
+    __syncthreads();
+    if (threadIdx.x == 0) s.go = 0;
+    cluster_sync();
+  }
   // Output: the kept set in ascending index order.
   if (g0) {
     int cnt = 0;
@@ -627,7 +706,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     mbar_wait(&s.bar_done, 0, reinterpret_cast<volatile int*>(&fresh), &g_diverse_err, 100000000ull);
   }
   tc_fence_before();
-  __syncthreads();
+  if (cs > 1) cluster_sync();
+  else __syncthreads();
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -658,10 +738,29 @@ cudaError_t launch_select_diverse(const SelectPlan& p, const SelectWorkspace& ws
   a.K = p.K;
   a.Kd = p.Kd;
   a.idx = idx;
+  // Four CTAs per image while their clusters surely run side by side (128 of
+  // the 152 SMs; a cluster's CTAs are of one SM group). Whole selector call, us,
+  // clusters of 1 / 4 / 8: 1 x 576 tokens 47.3 / 45.7 / 45.6, 16 x 576 110.3 /
+  // 109.7 / 120.2, 32 x 2880 765 / 753 / 832.
+  const int cs = p.B <= 32 ? 4 : 1;
   auto go = [&](auto kern, int threads) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDivSmem));
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, dim3(p.B), dim3(threads), kDivSmem, stream, a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.B * cs);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = kDivSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(cs);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, a);
   };
   // a token per thread where a block allows (the ranking of the pool and the
   // scatter around it, cycles per phase: 576 tokens on 144 threads of four each
