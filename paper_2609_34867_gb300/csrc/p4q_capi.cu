@@ -441,7 +441,7 @@ p4q_status run_linear_ws(const GemmArgs& g, void* ws, size_t ws_bytes, cudaStrea
   if (ws) {
     if (!aligned16(ws)) return P4Q_ERR_MISALIGNED;
     if (ws_bytes < gemm8_workspace_bytes(g.M, g.N, g.K)) return P4Q_ERR_WORKSPACE_TOO_SMALL;
-    if (gemm8_applies(g)) return from_cuda(counted(launch_w4a4_gemm8(g, ws, ws_bytes, stream), 3));
+    if (gemm8_applies(g)) return from_cuda(counted(launch_w4a4_gemm8(g, ws, ws_bytes, stream), 2));
   }
   return from_cuda(counted(launch_w4a4_gemm(g, stream)));
 }
@@ -492,7 +492,8 @@ p4q_status p4q_expand_codes(const uint8_t* q, int rows, int Kin, uint8_t* u, int
   if (rows == 0) return P4Q_OK;
   p4q_status st = check_device();
   if (st != P4Q_OK) return st;
-  return from_cuda(counted(launch_expand_codes(q, rows, Kin, u, sum_u, reinterpret_cast<cudaStream_t>(stream))));
+  return from_cuda(counted(launch_expand_codes(q, rows, Kin, u, sum_u, nullptr, 0, nullptr, nullptr,
+                                               reinterpret_cast<cudaStream_t>(stream))));
 }
 
 p4q_status p4q_w4a4_linear_expanded(const uint8_t* Xu, const int32_t* sum_xu, const float* s_a, int M, int Kin,

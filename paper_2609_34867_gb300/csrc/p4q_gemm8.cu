@@ -602,9 +602,8 @@ cudaError_t launch_gemm8(const GemmArgs& g, const uint8_t* a8, const int32_t* su
 cudaError_t launch_w4a4_gemm8(const GemmArgs& g, void* ws, size_t ws_bytes, cudaStream_t stream) {
   Ws8 w;
   if (!ws || ws_bytes < ws8_layout(g.M, g.N, g.K, ws, &w)) return cudaErrorInvalidValue;
-  cudaError_t e = launch_expand_codes(g.A, g.M, g.K, w.a8, w.sum_a, stream);
-  if (e != cudaSuccess) return e;
-  e = launch_expand_codes(g.B, g.N, g.K, w.b8, w.sum_b, stream);
+  cudaError_t e =
+      launch_expand_codes(g.B, g.N, g.K, w.b8, w.sum_b, g.A, g.M, w.a8, w.sum_a, stream);
   if (e != cudaSuccess) return e;
   return launch_gemm8(g, w.a8, w.sum_a, w.b8, w.sum_b, stream);
 }

@@ -170,3 +170,27 @@ def test_linear_expanded_matches_linear(p4q, dev):
     torch.cuda.synchronize()
     assert p4q.p4q_device_status() == 0
     assert torch.equal(Y.view(torch.int16), ref.view(torch.int16))
+
+
+@pytest.mark.parametrize("K", [128, 4096, 4224, 8192, 16384])
+@pytest.mark.parametrize("off", [0, 16])
+def test_expansion_alignments(p4q, dev, K, off):
+    """32-byte stores where the outputs allow, 16-byte stores otherwise: the
+    expansion alone (rows of every size class) and both operands in a workspace."""
+    rng = np.random.default_rng(K + off)
+    M, N = 515, 259 + 5
+    a, w = _packed(rng, M, K), _packed(rng, N, K)
+    da, dw = torch.from_numpy(a).to(dev), torch.from_numpy(w).to(dev)
+    buf = torch.empty(M * K + 16, dtype=torch.uint8, device=dev)
+    s = torch.empty(M, dtype=torch.int32, device=dev)
+    p4q.p4q_expand_codes(da, buf[off:off + M * K].view(M, K), s)
+    n = p4q.linear_workspace(M, N, K, dev).numel()
+    acc = p4q.w4a4_gemm_s32_ws(da, dw, torch.empty(n + 16, dtype=torch.uint8, device=dev)[off:off + n])
+    torch.cuda.synchronize()
+    assert p4q.p4q_device_status() == 0
+    v = oracle.unpack_codes(a).astype(np.int32) + 8
+    x = v.reshape(M, -1, 4, 2)
+    expect = np.concatenate([x[..., 0], x[..., 1]], axis=2).reshape(M, -1)
+    assert np.array_equal(buf[off:off + M * K].view(M, K).cpu().numpy().astype(np.int32), expect)
+    assert np.array_equal(s.cpu().numpy(), v.sum(axis=1))
+    assert np.array_equal(acc.cpu().numpy(), oracle.gemm_s32(oracle.unpack_codes(a), oracle.unpack_codes(w)))
