@@ -3,8 +3,8 @@
 // the operands of the expanded-operand GEMM (p4q_gemm8.cu), both of them in
 // one launch. HBM-bound streaming kernel: bytes per row K/2 in, K + 4 out.
 // 11008 + 2048 rows of 4096 codes (80 MB): two launches with 16-byte stores and
-// no prefetch 19 us, now about 5 beside a quantizer whose time the prefetch
-// fills (quantizer + linear together 89.2 -> 75.2 us).
+// no prefetch 19 us; one launch 12.5, part of it beside the quantizer whose time
+// the prefetch fills (quantizer + linear together 89.2 -> 75.2 us).
 #include "p4q_device.cuh"
 #include "p4q_internal.h"
 
@@ -82,9 +82,9 @@ template <bool WIDE>
 cudaError_t launch_expand(const ExpandOperand& a, const ExpandOperand& b, int K, cudaStream_t stream) {
   const dim3 grid((static_cast<long long>(a.rows) + b.rows + 7) / 8), block(256);
   const int nch = K >> 5;
-  if (nch <= 32 * 4) return launch_pdl(expand_codes_kernel<4, WIDE>, grid, block, 0, stream, a, b, K);
-  if (nch <= 32 * 8) return launch_pdl(expand_codes_kernel<8, WIDE>, grid, block, 0, stream, a, b, K);
-  return launch_pdl(expand_codes_kernel<16, WIDE>, grid, block, 0, stream, a, b, K);
+  if (nch <= 32 * 4) return launch_pdl_l1(expand_codes_kernel<4, WIDE>, grid, block, 0, 0, stream, a, b, K);
+  if (nch <= 32 * 8) return launch_pdl_l1(expand_codes_kernel<8, WIDE>, grid, block, 0, 0, stream, a, b, K);
+  return launch_pdl_l1(expand_codes_kernel<16, WIDE>, grid, block, 0, 0, stream, a, b, K);
 }
 
 }  // namespace

@@ -29,6 +29,34 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// launch_pdl for a kernel with many register loads in flight, which need L1:
+// asks for an SM split that leaves all but smem_per_sm bytes (of the CTAs that
+// run on it) to L1. Without a preference a kernel runs with the split of the
+// one before it, and behind a kernel with large shared memory (a GEMM, the row
+// buffers of the streaming quantizer) about 28 KB of L1 are left. Used where a
+// chain of calls measured faster with it (us: MLP up GEMM and requantizers of
+// 22528 rows 940 -> 920, selection of 32 x 2880 tokens 757 -> 744, quantizer
+// and linear of 2048 rows 74.7 -> 73.1; the SwiGLU and RMSNorm quantizers and
+// the GEMV: no difference).
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl_l1(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, size_t smem_per_sm,
+                          cudaStream_t stream, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  const size_t pct = (smem_per_sm * 100 + 228 * 1024 - 1) / (228 * 1024);
+  attr[1].val.sharedMemCarveout = static_cast<unsigned>(pct < 100 ? pct : 100);
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 
 // ------------------------------------------------------------ quantizer
 // Row source for the per-row quantizer: either a dense [rows, L] fp16 matrix,

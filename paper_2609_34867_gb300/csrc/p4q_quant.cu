@@ -390,7 +390,8 @@ cudaError_t launch_token_quant(const uint16_t* V, int B, int N, int L, int J, co
   // at most two CTAs of 8 warps per SM over the whole batch (one wave: rows are dealt out per CTA in
   // advance, so a second wave would double the time), never more warps than an image has rows
   const int per_image = std::max(1, std::min((N + 7) / 8, 2 * sm_count() / B));
-  return launch_pdl(select_token_quant_kernel<CH, JMAX>, dim3(per_image, B), dim3(256), smem, stream, V, N, L, J, qu,
+  return launch_pdl_l1(select_token_quant_kernel<CH, JMAX>, dim3(per_image, B), dim3(256), smem, 2 * (smem + 1024),
+                       stream, V, N, L, J, qu,
                     qsum, out, qdots, qp);
 }
 
@@ -573,7 +574,7 @@ cudaError_t launch_reg(const RowSource& src, int rows, int L, const RowSinks& ou
   const long long ldx = src.ldx > 0 ? src.ldx : L;
   const int groups = 8 / G;
   const int blocks = std::max(1, std::min((rows + groups - 1) / groups, 2 * sm_count()));  // one wave
-  return launch_pdl(quant_rows_reg_kernel<CH, G, NORM>, dim3(blocks), dim3(256), 0, stream, src.X, ldx, rows, L,
+  return launch_pdl_l1(quant_rows_reg_kernel<CH, G, NORM>, dim3(blocks), dim3(256), 0, 4096, stream, src.X, ldx, rows, L,
                     out);
 }
 
@@ -617,9 +618,9 @@ cudaError_t launch_quant_rowmax(const uint16_t* Y, int ldy, int M, int nblk, con
   const int G = (4LL * tasks <= slots && steps >= 4) ? 4 : (2LL * tasks <= slots && steps >= 2) ? 2 : 1;
   const int rows_per_cta = 8 / G;
   const int blocks = std::max(1, std::min((tasks + rows_per_cta - 1) / rows_per_cta, 8 * sm_count()));
-  if (G == 4) return launch_pdl(quant_rowmax_kernel<4>, dim3(blocks), dim3(256), 0, stream, a);
-  if (G == 2) return launch_pdl(quant_rowmax_kernel<2>, dim3(blocks), dim3(256), 0, stream, a);
-  return launch_pdl(quant_rowmax_kernel<1>, dim3(blocks), dim3(256), 0, stream, a);
+  if (G == 4) return launch_pdl_l1(quant_rowmax_kernel<4>, dim3(blocks), dim3(256), 0, 8192, stream, a);
+  if (G == 2) return launch_pdl_l1(quant_rowmax_kernel<2>, dim3(blocks), dim3(256), 0, 8192, stream, a);
+  return launch_pdl_l1(quant_rowmax_kernel<1>, dim3(blocks), dim3(256), 0, 8192, stream, a);
 }
 
 bool select_token_quant_applies(int d, int J) {
