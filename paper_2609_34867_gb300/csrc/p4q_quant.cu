@@ -150,18 +150,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       uint32_t* q4 = out.codes ? reinterpret_cast<uint32_t*>(out.codes + static_cast<size_t>(row) * (L >> 1)) : nullptr;
       uint4* cp = out.copy ? reinterpret_cast<uint4*>(out.copy + static_cast<size_t>(row) * L) : nullptr;
       uint2* up = out.u ? reinterpret_cast<uint2*>(out.u + static_cast<size_t>(row) * L) : nullptr;
+      by_rounding(qr, [&](auto tie) {
 #pragma unroll 4
-      for (int c = gt; c < nch; c += kGroupThreads) {
-        const uint4 v = v4[c];
-        const Codes8 cd = (a != 0.0f) ? quant_chunk<NORM>(v, qr, n2) : Codes8{0u, 0u};
-        if (q4) q4[c] = packed4(cd);
-        if (cp) cp[c] = v;
-        if (up) {
-          const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
-          up[c] = make_uint2(eu, ou);
-          su = __dp4a(eu + ou, 0x01010101u, su);
+        for (int c = gt; c < nch; c += kGroupThreads) {
+          const uint4 v = v4[c];
+          const Codes8 cd = quant_chunk<NORM, decltype(tie)::value>(v, qr, n2);
+          if (q4) q4[c] = packed4(cd);
+          if (cp) cp[c] = v;
+          if (up) {
+            const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
+            up[c] = make_uint2(eu, ou);
+            su = __dp4a(eu + ou, 0x01010101u, su);
+          }
         }
-      }
+      });
     }
     int wn = 0, wu = 0;
     if (NORM) {
@@ -279,22 +281,33 @@ cudaError_t launch_norm(const RowSource& src, int rows, int L, const RowSinks& o
 // ---------------------------------------------------------------- selector token pass
 // The selector's fake-quantized tokens (the quantizer above with the squared
 // code norm and the expanded codes) with the Eq. 4 query dot products fused:
-// one warp per token row, the row held in registers (CH 16-byte chunks per
-// lane, all loads of a row in flight at once), the abs-max a warp reduction,
-// no shared-memory pass and no block barrier. CTA (x, b) takes rows of image
-// b only, so the image's J concept rows (expanded codes, written by the
-// concept pass before this launch) sit in shared memory and each chunk's
-// bytes u are multiplied into them by dp4a as they are produced: the exact
-// code dot product with concept j is sum u u_j - 8 sum u - 8 sum u_j + 64 L.
-// Rolling prefetch: as soon as a chunk is quantized its registers take the
-// same chunk of the warp's next row, so the next row's loads are in flight
-// during the rest of this row's work without more registers.
+// two warps per token row, the row held in registers (CH 16-byte chunks per
+// lane, all loads of a row in flight at once), no shared-memory pass. CTA
+// (x, b) takes rows of image b only, so the image's J concept rows (expanded
+// codes, written by the concept pass before this launch) sit in shared memory
+// and each chunk's bytes u are multiplied into them by dp4a as they are
+// produced: the exact code dot product with concept j is sum u u_j - 8 sum u -
+// 8 sum u_j + 64 L. Rolling prefetch: as soon as a chunk is quantized its
+// registers take the same chunk of the pair's next row, so the next row's
+// loads are in flight during the rest of this row's work without more
+// registers. One barrier of the pair per row: a row's sums are put together
+// after the next row's abs-max barrier.
+// Bound: memory, next to issue (about 60 instructions per chunk of 256 values).
+// 32 x 2880 rows of 5120 (1.4 GB, 208 us at the measured copy rate): 217 us;
+// with one warp per row (128 registers, 16 warps per SM) 232, with that and two
+// products per value 272.
+constexpr int kTokCtas = 3;  // per SM
+constexpr size_t kTokSmemThree = 72 * 1024;  // concept rows with three CTAs per SM
+
 template <int CH, int JMAX>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, kTokCtas)
     select_token_quant_kernel(const uint16_t* __restrict__ V, int N, int L, int J, const uint8_t* __restrict__ qu,
                               const int32_t* __restrict__ qsum, RowSinks out, float* __restrict__ qdots, int qp) {
   extern __shared__ __align__(16) uint8_t cq[];  // [J, L] the image's concept codes, expanded
+  __shared__ uint32_t red_max[2][8];             // by row parity and warp
+  __shared__ uint32_t red_sum[2][8][2 + JMAX];   // sums of u, of u^2 and of u u_j
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int grp = warp >> 1, gt = threadIdx.x & 63;
   pdl_wait();  // the concept codes come from the previous launch
   pdl_launch_dependents();
   if (JMAX > 0) {
@@ -303,21 +316,42 @@ __global__ void __launch_bounds__(256, 2)
     __syncthreads();
   }
   const int nch = L >> 3;
-  const int wpi = gridDim.x * (blockDim.x >> 5);  // warps per image
-  const int r_first = blockIdx.x * (blockDim.x >> 5) + warp;
+  const int step = gridDim.x * 4;  // pairs of warps per image
+  const int r_first = blockIdx.x * 4 + grp;
   uint4 v[CH];
   if (r_first < N) {
     const uint4* x = reinterpret_cast<const uint4*>(V + (static_cast<size_t>(b) * N + r_first) * L);
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
-      const int c = lane + 32 * i;
+      const int c = gt + 64 * i;
       v[i] = (c < nch) ? ldg_stream16(x + c) : make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  for (int r = r_first; r < N; r += wpi) {
+  // the first warp of the pair: the outputs of row r (sums of parity par, scale s)
+  auto finish = [&](int r, int par, float s) {
     const size_t row = static_cast<size_t>(b) * N + r;
-    const bool more = r + wpi < N;
-    const uint4* xn = reinterpret_cast<const uint4*>(V + (row + (more ? wpi : 0)) * L);  // the warp's next row
+    const int k = min(lane, 1 + JMAX);
+    const uint32_t mine = lane < 2 + J ? red_sum[par][warp][k] + red_sum[par][warp + 1][k] : 0u;
+    const int wu = static_cast<int>(__shfl_sync(0xFFFFFFFFu, mine, 0));
+    if (lane == 0) {
+      out.scale[row] = s;
+      out.sum_u[row] = wu;
+    } else if (lane == 1) {
+      // sum of squared codes (u - 8)^2 over the row's L codes, exactly
+      out.norm2[row] = static_cast<int>(mine) - 16 * wu + 64 * L;
+    } else if (JMAX > 0 && lane < 2 + J) {
+      // exact (|dot| <= 49 L < 2^24), so the float holds it exactly
+      const int j = lane - 2;
+      const int dot = static_cast<int>(mine) - 8 * wu - 8 * qsum[b * J + j] + 64 * L;
+      qdots[row * qp + j] = static_cast<float>(dot);
+    }
+  };
+  int par = 0, prev = -1;
+  float prev_s = 0.0f;
+  for (int r = r_first; r < N; r += step, par ^= 1) {  // uniform across the pair
+    const size_t row = static_cast<size_t>(b) * N + r;
+    const bool more = r + step < N;
+    const uint4* xn = reinterpret_cast<const uint4*>(V + (row + (more ? step : 0)) * L);  // the pair's next row
     uint32_t m = 0;  // per-halfword max of |x| bit patterns
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
@@ -326,7 +360,11 @@ __global__ void __launch_bounds__(256, 2)
       m = __vmaxu2(m, v[i].z & 0x7FFF7FFFu);
       m = __vmaxu2(m, v[i].w & 0x7FFF7FFFu);
     }
-    const uint32_t mm = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+    const uint32_t wm = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+    if (lane == 0) red_max[par][warp] = wm;
+    named_bar_sync(1 + grp, 64);
+    const uint32_t mm = max(wm, red_max[par][warp ^ 1]);
+    if (prev >= 0 && (warp & 1) == 0) finish(prev, par ^ 1, prev_s);
     const float a = __half2float(__ushort_as_half(static_cast<unsigned short>(mm)));
     const QRow qr = quant_row(a);
     float2 n2 = make_float2(0.0f, 0.0f);  // unused: the norm comes from the expanded codes
@@ -335,44 +373,44 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
     for (int j = 0; j < (JMAX > 0 ? JMAX : 1); ++j) dq[j] = 0;
     uint2* up = reinterpret_cast<uint2*>(out.u + row * L);
+    by_rounding(qr, [&](auto tie) {
 #pragma unroll
-    for (int i = 0; i < CH; ++i) {
-      const int c = lane + 32 * i;
-      if (c < nch) {
-        const Codes8 cd = (a != 0.0f) ? quant_chunk<false>(v[i], qr, n2) : Codes8{0u, 0u};
-        if (more) v[i] = ldg_stream16(xn + c);
-        const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
-        up[c] = make_uint2(eu, ou);
-        su = __dp4a(eu + ou, 0x01010101u, su);
-        uu = __dp4a(eu, eu, __dp4a(ou, ou, uu));
+      for (int i = 0; i < CH; ++i) {
+        const int c = gt + 64 * i;
+        if (c < nch) {
+          const Codes8 cd = quant_chunk<false, decltype(tie)::value>(v[i], qr, n2);
+          if (more) v[i] = ldg_stream16(xn + c);
+          const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
+          up[c] = make_uint2(eu, ou);
+          su = __dp4a(eu + ou, 0x01010101u, su);
+          uu = __dp4a(eu, eu, __dp4a(ou, ou, uu));
 #pragma unroll
-        for (int j = 0; j < JMAX; ++j) {
-          if (j < J) {
-            const uint2 w = *reinterpret_cast<const uint2*>(cq + static_cast<size_t>(j) * L + 8 * c);
-            dq[j] = __dp4a(eu, w.x, __dp4a(ou, w.y, dq[j]));
+          for (int j = 0; j < JMAX; ++j) {
+            if (j < J) {
+              const uint2 w = *reinterpret_cast<const uint2*>(cq + static_cast<size_t>(j) * L + 8 * c);
+              dq[j] = __dp4a(eu, w.x, __dp4a(ou, w.y, dq[j]));
+            }
           }
         }
       }
-    }
-    const int wu = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, su));
-    // sum of squared codes (u - 8)^2 over the row's L codes, exactly
-    const int wn = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, uu)) - 16 * wu + 64 * L;
+    });
+    su = __reduce_add_sync(0xFFFFFFFFu, su);
+    uu = __reduce_add_sync(0xFFFFFFFFu, uu);
+    if (lane == 0) red_sum[par][warp][0] = su;
+    if (lane == 0) red_sum[par][warp][1] = uu;
 #pragma unroll
     for (int j = 0; j < JMAX; ++j) {
       if (j < J) {
-        const int p = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, dq[j]));
-        if (lane == j) {
-          // exact (|dot| <= 49 L < 2^24), so the float holds it exactly
-          const int dot = p - 8 * wu - 8 * qsum[b * J + j] + 64 * L;
-          qdots[row * qp + j] = static_cast<float>(dot);
-        }
+        const uint32_t p = __reduce_add_sync(0xFFFFFFFFu, dq[j]);
+        if (lane == 0) red_sum[par][warp][2 + j] = p;
       }
     }
-    if (lane == 0) {
-      out.scale[row] = (a != 0.0f) ? qr.s : 0.0f;
-      out.norm2[row] = wn;
-      out.sum_u[row] = wu;
-    }
+    prev = r;
+    prev_s = (a != 0.0f) ? qr.s : 0.0f;
+  }
+  if (prev >= 0) {
+    named_bar_sync(1 + grp, 64);
+    if ((warp & 1) == 0) finish(prev, par ^ 1, prev_s);
   }
 }
 
@@ -387,12 +425,13 @@ cudaError_t launch_token_quant(const uint16_t* V, int B, int N, int L, int J, co
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  // at most two CTAs of 8 warps per SM over the whole batch (one wave: rows are dealt out per CTA in
-  // advance, so a second wave would double the time), never more warps than an image has rows
-  const int per_image = std::max(1, std::min((N + 7) / 8, 2 * sm_count() / B));
-  return launch_pdl_l1(select_token_quant_kernel<CH, JMAX>, dim3(per_image, B), dim3(256), smem, 2 * (smem + 1024),
-                       stream, V, N, L, J, qu,
-                    qsum, out, qdots, qp);
+  // at most as many CTAs as run at once over the whole batch (one wave: rows are dealt out per CTA in
+  // advance, so a second wave would double the time), never more pairs of warps than an image has rows
+  const int ctas = smem <= kTokSmemThree ? kTokCtas : 2;
+  const int per_image = std::max(1, std::min((N + 3) / 4, ctas * sm_count() / B));
+  return launch_pdl_l1(select_token_quant_kernel<CH, JMAX>, dim3(per_image, B), dim3(256), smem,
+                          ctas * (smem + 3 * 1024), stream, V, N, L, J,
+                    qu, qsum, out, qdots, qp);
 }
 
 // ---------------------------------------------------------------- known row abs-max
@@ -400,11 +439,10 @@ cudaError_t launch_token_quant(const uint16_t* V, int B, int N, int L, int J, co
 // known (the GEMM's row-max epilogue): no abs-max pass, no reduction before
 // the codes, so G warps stream a block row in 256-element steps (one 16-byte
 // chunk per lane, steps interleaved over the G warps, kRmUnroll in flight per
-// warp) and only the row sum of the expanded codes is reduced at the end. The
-// pass is issue-bound (about 14 instructions per code at a quarter of the
-// warp slots), so a few thousand rows (the short sequences) take G = 2 or 4
-// warps per row to fill the GPU; G = 1 otherwise. Same arithmetic as
-// quant_rows_kernel (s = a / 7, quant_chunk), so the same codes and scales.
+// warp) and only the row sum of the expanded codes is reduced at the end. A few
+// thousand rows (the short sequences) take G = 2 or 4 warps per row to fill the
+// GPU; G = 1 otherwise. Same arithmetic as quant_rows_kernel (s = a / 7,
+// quant_chunk), so the same codes and scales.
 struct RowmaxArgs {
   const uint16_t* Y;
   int ldy, M, nblk;
@@ -449,18 +487,20 @@ __global__ void __launch_bounds__(256, 4) quant_rowmax_kernel(RowmaxArgs a) {
         const int j = j0 + k * G;
         v[k] = (j < steps) ? ldg_stream16(x + j * 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
       }
+      by_rounding(qr, [&](auto tie) {
 #pragma unroll
-      for (int k = 0; k < kRmUnroll; ++k) {
-        const int j = j0 + k * G;
-        if (j < steps) {
-          const int c = j * 32 + lane;
-          const Codes8 cd = (amax != 0.0f) ? quant_chunk<false>(v[k], qr, n2) : Codes8{0u, 0u};
-          if (q4) q4[c] = packed4(cd);
-          const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
-          up[c] = make_uint2(eu, ou);
-          su = __dp4a(eu + ou, 0x01010101u, su);
+        for (int k = 0; k < kRmUnroll; ++k) {
+          const int j = j0 + k * G;
+          if (j < steps) {
+            const int c = j * 32 + lane;
+            const Codes8 cd = quant_chunk<false, decltype(tie)::value>(v[k], qr, n2);
+            if (q4) q4[c] = packed4(cd);
+            const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
+            up[c] = make_uint2(eu, ou);
+            su = __dp4a(eu + ou, 0x01010101u, su);
+          }
         }
-      }
+      });
     }
     uint32_t wu = __reduce_add_sync(0xFFFFFFFFu, su);
     if (G > 1) {
@@ -532,19 +572,21 @@ __global__ void __launch_bounds__(256, 2)
     uint32_t su = 0, uu = 0;
     uint32_t* q4 = out.codes ? reinterpret_cast<uint32_t*>(out.codes + static_cast<size_t>(r) * (L >> 1)) : nullptr;
     uint2* up = out.u ? reinterpret_cast<uint2*>(out.u + static_cast<size_t>(r) * L) : nullptr;
+    by_rounding(qr, [&](auto tie) {
 #pragma unroll
-    for (int i = 0; i < CH; ++i) {
-      const int c = gt + 32 * G * i;
-      if (c < nch) {
-        const Codes8 cd = (a != 0.0f) ? quant_chunk<false>(v[i], qr, n2) : Codes8{0u, 0u};
-        if (more) v[i] = ldg_stream16(xn + c);
-        if (q4) q4[c] = packed4(cd);
-        const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
-        if (up) up[c] = make_uint2(eu, ou);
-        su = __dp4a(eu + ou, 0x01010101u, su);
-        if (NORM) uu = __dp4a(eu, eu, __dp4a(ou, ou, uu));
+      for (int i = 0; i < CH; ++i) {
+        const int c = gt + 32 * G * i;
+        if (c < nch) {
+          const Codes8 cd = quant_chunk<false, decltype(tie)::value>(v[i], qr, n2);
+          if (more) v[i] = ldg_stream16(xn + c);
+          if (q4) q4[c] = packed4(cd);
+          const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
+          if (up) up[c] = make_uint2(eu, ou);
+          su = __dp4a(eu + ou, 0x01010101u, su);
+          if (NORM) uu = __dp4a(eu, eu, __dp4a(ou, ou, uu));
+        }
       }
-    }
+    });
     int wu = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, su));
     int wuu = NORM ? static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, uu)) : 0;
     if (G > 1) {
@@ -639,11 +681,11 @@ cudaError_t launch_select_token_quant(const uint16_t* V, int B, int N, int d, in
     if (J <= 4) return launch_token_quant<C, 4>(V, B, N, d, J, qu, qsum, out, qdots, qp, stream);
     return launch_token_quant<C, 16>(V, B, N, d, J, qu, qsum, out, qdots, qp, stream);
   };
-  if (ch <= 4) return go(std::integral_constant<int, 4>());
-  if (ch <= 8) return go(std::integral_constant<int, 8>());
-  if (ch <= 12) return go(std::integral_constant<int, 12>());
-  if (ch <= 16) return go(std::integral_constant<int, 16>());
-  return go(std::integral_constant<int, 20>());
+  if (ch <= 4) return go(std::integral_constant<int, 2>());
+  if (ch <= 8) return go(std::integral_constant<int, 4>());
+  if (ch <= 12) return go(std::integral_constant<int, 6>());
+  if (ch <= 16) return go(std::integral_constant<int, 8>());
+  return go(std::integral_constant<int, 10>());
 }
 
 

@@ -31,9 +31,9 @@
 // Bound: instruction issue. The splits run two values at a time
 // (add/fma.rn.f32x2), t w is one fp16 multiplication (its exact product
 // rounded once, as the fp32 product rounded to fp16 is), the maxima are taken
-// on fp16 pairs and the codes from the bracketing products of p4q_codes.cuh.
-// Measured (us; one value at a time before): 2048 x 4096 9.4 (14.2) = 3.1 TB/s,
-// 2048 x 5120 13.0 (21.3), 16000 x 5120 79 (149).
+// on fp16 pairs and the codes take one product per value (p4q_codes.cuh).
+// Measured (us; one value at a time before): 2048 x 4096 8.5 (14.2) = 3.4 TB/s;
+// with two products per value 2048 x 5120 13.0 (21.3), 16000 x 5120 79 (149).
 #include <cuda_fp16.h>
 
 #include "p4q.h"
@@ -179,20 +179,22 @@ __global__ void __launch_bounds__(THREADS)
   uint2* up2 = EXPANDED ? reinterpret_cast<uint2*>(Xu + static_cast<size_t>(row) * K) : nullptr;
   uint32_t su = 0;
   float2 n2 = make_float2(0.0f, 0.0f);  // unused
+  by_rounding(q, [&](auto tie) {
 #pragma unroll
-  for (int j = 0; j < MAXC; ++j) {
-    const int c = t + j * THREADS;
-    if (c < nch) {
-      const Codes8 cd = (a != 0.0f) ? quant_chunk<false>(xv[j], q, n2) : Codes8{0u, 0u};
-      q4[c] = packed4(cd);
-      if (EXPANDED) {
-        // the even values, then the odd ones, offset by 8 (the GEMM's order)
-        const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
-        up2[c] = make_uint2(eu, ou);
-        su = __dp4a(eu + ou, 0x01010101u, su);
+    for (int j = 0; j < MAXC; ++j) {
+      const int c = t + j * THREADS;
+      if (c < nch) {
+        const Codes8 cd = quant_chunk<false, decltype(tie)::value>(xv[j], q, n2);
+        q4[c] = packed4(cd);
+        if (EXPANDED) {
+          // the even values, then the odd ones, offset by 8 (the GEMM's order)
+          const uint32_t eu = expanded_even(cd), ou = expanded_odd(cd);
+          up2[c] = make_uint2(eu, ou);
+          su = __dp4a(eu + ou, 0x01010101u, su);
+        }
       }
     }
-  }
+  });
   if (t == 0) s_a[row] = (a != 0.0f) ? s : 0.0f;
   if (EXPANDED) {
     const int ws = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, su));

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (MAXC <= 3 ? 4 : 2) 
   float a = 0.0f;
 #pragma unroll
   for (int w = 0; w < THREADS / 32; ++w) a = fmaxf(a, wmax[w]);
-  QRow q = quant_row(a);
+  QRowF q = quant_row_f(a);
   const float s = q.s;
   q.s = -q.s;  // the values are held negated
   q.ip = -q.ip;
