@@ -10,7 +10,7 @@
 // over its int32 tiles; in Gram mode a row pass over the token-pair GEMM)
 // as m. After that no cosine row of the whole image is ever formed. The kernel holds, for every free token, a
 // lower bound of m (exact up to the first ex picks) and runs in phases:
-//   1. pool: the 128 smallest free (bound, token) pairs (block radix select);
+//   1. pool: the 128 smallest free (bound, token) pairs (block_take_top);
 //      tau = the largest of them. Every token outside the pool has a pair
 //      above tau, and its true pair is at least its bound's.
 //   2. the pool's exact cosines: code dot products of the pool rows with the

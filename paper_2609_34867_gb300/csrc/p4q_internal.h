@@ -193,7 +193,7 @@ size_t block_mse_workspace_bytes(int B);
 // off: host array of B + 1 row offsets (validated by the caller).
 cudaError_t launch_block_mse(const uint16_t* Yq, long long ldq, const uint16_t* Yf, long long ldf, const int32_t* off,
                              int B, int d, double* partial, float* e, float* L, cudaStream_t stream);
-// Top-K sets of two score rows per sample and their intersection (selector's radix select).
+// Top-K sets of two score rows per sample and their intersection (the selector's ranking).
 cudaError_t launch_topk_replacement(const float* s_ref, const float* s_alt, int B, int N, int K, int32_t* inter,
                                     float* rho, cudaStream_t stream);
 

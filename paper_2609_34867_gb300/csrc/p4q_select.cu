@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* __restrict_
 
 // ---------------------------------------------------------------- Top-K replacement ratio
 // App. A, Eq. 9: per sample, the Top-K sets of two score rows over the same N
-// tokens (ties to the lower index, the selector's radix select) and the size
+// tokens (ties to the lower index, the selector's ranking) and the size
 // of their intersection; rho = 1 - |T_ref & T_alt| / K. One CTA per sample,
 // token i = kPer * threadIdx.x + e.
 // Order key of a score with -0 and +0 equal (they tie, and the lower index wins).
