@@ -89,7 +89,9 @@ uint64_t p4q_launch_count(void);
  *     on the CUDA cores: the packed weights are read once); for few rows (M
  *     <= 128 and M * ceil(N / 128) <= 8192) a kernel with the weights on the
  *     tensor cores' row side and k split over a cluster; CTA-pair kernel for
- *     fp16 outputs with M >= 256 and N >= 256; single-CTA kernel otherwise;
+ *     fp16 outputs with M >= 256 and N >= 256, or with N >= 1024 from M = 129
+ *     (from M = 65 while ceil(N / 256) <= the CTA pairs of the GPU);
+ *     single-CTA kernel otherwise;
  *   1 single-CTA kernel only;
  *   2 CTA-pair kernel whenever N >= 256 (also for int32 outputs);
  *   3 like 0, and the workspace entry points take the expanded-operand path

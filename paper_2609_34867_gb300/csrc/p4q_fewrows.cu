@@ -520,12 +520,20 @@ cudaError_t launch_out(const GemmArgs& g, cudaStream_t stream) {
 // Up to 128 rows, and fewer for more weight rows: every CTA unpacks its share
 // of the activations, and with M * ceil(N / 128) past 8192 that costs more
 // than the in-kernel unpack of p4q_gemm.cu on 256-row weight tiles (measured,
-// us, this kernel / that one: 64 x 12288 x 4096 21.7 / 29.0, 64 x 22016 x 4096
-// 34.2 / 29.6, 96 x 12288 x 4096 35.0 / 29.7, 128 x 4096 x 4096 13.3 / 30.5).
+// us, this kernel / that one: 64 x 12288 x 4096 21.7 / 26.0, 64 x 22016 x 4096
+// 34.2 / 29.6, 96 x 12288 x 4096 35.0 / 25.9, 128 x 4096 x 4096 13.3 / 25.4).
+// Past K = 8192 only where the activations are one row tile of the CTA's shared
+// memory: a second tile reads the weights again, against that file's CTA pairs
+// (128 x 5120 x 5120 27.9 / 29.3, 96 x 5120 x 13824 45.3 / 62.2, 128 x 4096 x
+// 11008 56.2 / 51.5, 128 x 5120 x 13824 74.6 / 62.2).
 bool fewrows_applies(const GemmArgs& g) {
+  const int nkb = (g.K / kBK + kMaxCluster - 1) / kMaxCluster;
+  const bool one_tile = g.M <= kMaxRowTile && 1024 + few_x_bytes(g.M, (g.M + 16) / 16 * 16, (g.M + 8) / 8 * 8, nkb) +
+                                                      2 * kPairBytes <= kSmemMax;
+  const bool pairs_serve = g.out == GemmOut::kHalf && g.N >= 1024 && (g.N + 255) / 256 <= num_sms() / 2;
   return (g.out == GemmOut::kHalf || g.out == GemmOut::kS32) && g.batch == 1 && g.M >= 1 && g.M <= 128 &&
          static_cast<long long>(g.M) * ((g.N + kTileN - 1) / kTileN) <= 8192 && g.N % 2 == 0 && g.K % kBK == 0 &&
-         (g.d_pitch == 0 || g.d_pitch == g.N);
+         (g.d_pitch == 0 || g.d_pitch == g.N) && (g.K <= 8192 || one_tile || !pairs_serve);
 }
 
 cudaError_t launch_fewrows(const GemmArgs& g, cudaStream_t stream) {

@@ -1073,8 +1073,16 @@ cudaError_t launch_w4a4_gemm(const GemmArgs& g, cudaStream_t stream) {
   // weights on the MMAs' row side, k split over clusters (automatic mode only)
   if (g_pair_mode == -1 && gemv_applies(g)) return launch_gemv(g, stream);
   if (g_pair_mode == -1 && fewrows_applies(g)) return launch_fewrows(g, stream);
+  // fp16 outputs on CTA pairs: from 256 rows; from 129 rows where the single-CTA
+  // kernel takes 256-column tiles too; and for 65 - 128 rows while the column
+  // tiles are one round of the pairs (the single CTAs, twice as many, then still
+  // run one round where the pairs need two). Measured (us, single / pair): 160 x
+  // 256 x 4096 (N x K) 21.7 / 24.6, 160 x 1024 x 4096 29.0 / 25.0, 160 x 4096 x
+  // 11008 71.1 / 51.5, 160 x 27648 x 5120 73.3 / 52.6, 96 x 12288 x 4096 29.7 /
+  // 25.9, 96 x 22016 x 4096 30.6 / 43.7, 33 x 12288 x 4096 33.4 / 42.5.
+  const bool pair_rows = g.M >= 256 || (g.N >= 1024 && (g.M > 128 || (g.M > 64 && (g.N + 255) / 256 <= num_sms() / 2)));
   const bool pair_ok = g.M > 0 && g.N >= 256 && g.batch > 0 && g_pair_mode != 0 &&
-                       (g_pair_mode == 1 || (g.M >= 256 && g.out == GemmOut::kHalf));
+                       (g_pair_mode == 1 || (pair_rows && g.out == GemmOut::kHalf));
   if (pair_ok && g.out == GemmOut::kHalf) return launch_pair<0>(g, stream);
   if (pair_ok && g.out == GemmOut::kS32) return launch_pair<1>(g, stream);
   // exact dot products of large token sets (the selector's Gram matrices):

@@ -156,7 +156,7 @@ cudaError_t launch_fewrows(const GemmArgs& g, cudaStream_t stream);
 unsigned int fewrows_read_and_clear_error();
 
 // Which GEMM kernel serves fp16 / int32 outputs: -1 automatic (the
-// weight-streaming kernel for M <= 2, the few-rows kernel, the CTA-pair kernel for large fp16
+// weight-streaming kernel for M <= 2, the few-rows kernel, the CTA-pair kernel for larger fp16
 // linears), 0 single-CTA only, 1 CTA-pair whenever the shape allows (N >= 256).
 void set_gemm_pair_mode(int mode);
 // Expanded-operand path: 0 automatic (M >= 512), 1 never, 2 whenever a workspace is given.

@@ -35,3 +35,12 @@ def test_fewrows_bit_exact(p4q, dev, M, N, K):
     assert np.array_equal(acc.cpu().numpy(), ref)
     y = (ref.astype(np.float32) * sa[:, None]) * sw[None, 1:]
     assert np.array_equal(Y.cpu().numpy(), y.astype(np.float16))
+
+
+@pytest.mark.parametrize("M,N,K", [(128, 8448, 128), (65, 16384, 256), (65, 19712, 128), (64, 16640, 128),
+                                   (129, 1016, 384), (129, 1024, 384), (255, 1032, 640), (160, 4096, 11008),
+                                   (109, 1032, 13824), (112, 1032, 13824), (128, 1032, 11008), (128, 264, 8320),
+                                   (95, 1024, 16384), (96, 1024, 16384)])
+def test_dispatch_edges(p4q, dev, M, N, K):
+    """Around the lines between the few-rows kernel, the CTA pairs and the single CTAs."""
+    test_fewrows_bit_exact(p4q, dev, M, N, K)
