@@ -436,8 +436,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool pending = false;
     uint8_t* box = smem + kOffO + (warp - 2) * 4096;
     auto epilogue = [&](bool live) {
-      float* rl = red + 2 * kBQ;  // row sums of the halves (rewritten one unit later, after
-                                  // the partner has passed the chunk barriers in between)
+      // Row sums of the halves. Both warps of the quad pass a barrier between
+      // this unit's reads of them and the next unit's writes: that of a chunk
+      // in between, or the one before the last unit's output.
+      float* rl = red + 2 * kBQ;
       rl[half * kBQ + r] = e_l;
       if (lane == 0) bulk_wait_group_read<0>();  // the last unit's store has read the box
       named_bar_sync(1 + quad, 64);
@@ -610,6 +612,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     if (pending) {  // the last unit
+      // (of one chunk only, it follows the output of the unit before at once:
+      // the partner may still be reading that one's row sums)
+      named_bar_sync(1 + quad, 64);
       const int jl = it.j - 1;
       if (ok && jl >= 0) ok = mbar_wait_all(&br.pv_done[jl & 1], (jl >> 1) & 1, abort_flag, &g_attn_err);
       tc_fence_after();

@@ -121,3 +121,24 @@ def test_attention_units_and_moving_maxima(p4q, dev, B, m, H, Hkv, scale):
     q, k, v = _inputs(B, m, H, Hkv, seed=m, qscale=scale)
     got = _run(p4q, dev, q, k, v, B, m, H, Hkv)
     _check(got, oracle.causal_attention(q, k, v, B, m, H, Hkv, DH), v, B, m, H, Hkv)
+
+
+@pytest.mark.parametrize("B,m", [(30, 100), (9, 250)])
+def test_attention_last_units_of_one_chunk(p4q, dev, B, m):
+    """A CTA's last unit of a single chunk is written straight after the unit
+    before it: each keeps its own row sums. Values of 1 make every output 1 up to
+    the weights' rounding (2^-11 each) and the output's, 5.2e-4 x 2 + 1e-5 as
+    above; the heads' row sums alternate between the row's length (equal keys)
+    and about 1 (one key dominates), so a sum of the wrong unit shows."""
+    H = 40
+    q, k, _ = _inputs(B, m, H, H, seed=B)
+    q.reshape(B * m, H, DH)[:, 0::2] = 0
+    q.reshape(B * m, H, DH)[:, 1::2] *= np.float16(8)
+    v = np.ones((B * m, H * DH), np.float16)
+    Q, K, V = (torch.from_numpy(a).to(dev) for a in (q, k, v))
+    O = torch.empty((20, B * m, H * DH), dtype=torch.float16, device=dev)
+    for o in O:
+        p4q.p4q_causal_attention(Q, K, V, o, B, m, H, H)
+    torch.cuda.synchronize()
+    assert p4q.p4q_device_status() == 0
+    assert float((O.float() - 1).abs().max()) <= 5.2e-4 * 2 + 1e-5
