@@ -42,8 +42,7 @@ __device__ __forceinline__ double block_sum_f64(double v, double* red) {
 }
 
 __global__ void __launch_bounds__(kMseThreads)
-    mse_partial_kernel(const __half* __restrict__ Yq, const __half* __restrict__ Yf, const MseParams p,
-                       double* __restrict__ partial) {
+    mse_partial_kernel(const __half* Yq, const __half* Yf, const MseParams p, double* partial) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ double red[kMseThreads / 32];
@@ -62,8 +61,8 @@ __global__ void __launch_bounds__(kMseThreads)
       if (i < items) {
         const int rr = i / nch, k = i - rr * nch;
         const size_t r = static_cast<size_t>(r0 + c + rr * C);
-        a[u] = __ldg(reinterpret_cast<const uint4*>(Yq + r * p.ldq) + k);
-        f[u] = __ldg(reinterpret_cast<const uint4*>(Yf + r * p.ldf) + k);
+        a[u] = reinterpret_cast<const uint4*>(Yq + r * p.ldq)[k];
+        f[u] = reinterpret_cast<const uint4*>(Yf + r * p.ldf)[k];
       } else {
         a[u] = make_uint4(0u, 0u, 0u, 0u);
         f[u] = a[u];
@@ -87,8 +86,7 @@ __global__ void __launch_bounds__(kMseThreads)
 }
 
 __global__ void __launch_bounds__(kMseThreads)
-    mse_final_kernel(const double* __restrict__ partial, int C, const MseParams p, float* __restrict__ e,
-                     float* __restrict__ L) {
+    mse_final_kernel(const double* partial, int C, const MseParams p, float* e, float* L) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ double red[kMseThreads / 32];

@@ -37,6 +37,13 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 // completed, which that one does only after its own wait, so what a kernel
 // reads is still complete; and the weights of a linear are on their way while
 // the linear before its quantizer still runs.
+// So a kernel may start before the one two ahead of it has read a buffer that
+// the one in between rewrites (codes of one buffer, quantized again for each
+// linear): what it reads from the stream's earlier kernels is not read-only for
+// its lifetime. Kernels therefore read with ordinary loads, which see everything
+// before pdl_wait(), and not through the read-only path (ld.global.nc, __ldg,
+// const __restrict__ parameters), which may return an older line of L1. (The
+// one exception, ldg_readonly16, states why its data is read-only.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -205,8 +212,19 @@ __device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap* map, int c
                : "memory");
 }
 
-// 16-byte global load that bypasses L1 allocation (data is consumed once per CTA).
+// 16-byte global load that bypasses L1 allocation (data is consumed once per
+// CTA).
 __device__ __forceinline__ uint4 ldg_stream16(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// ldg_stream16 through the read-only path, for data that no kernel may still be
+// writing when this one launches (see programmatic dependent launch above).
+__device__ __forceinline__ uint4 ldg_readonly16(const void* p) {
   uint4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)

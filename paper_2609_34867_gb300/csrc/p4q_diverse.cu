@@ -249,7 +249,7 @@ __device__ __forceinline__ void cand_cosines(const DivArgs& a, int b, int npool,
 #pragma unroll
       for (int k = 0; k < kPoolPer; ++k) {
         const int f = lane + 32 * k;
-        v[j][k] = f < npool && f >= e ? __ldg(row + fc[k]) : 0.0f;
+        v[j][k] = f < npool && f >= e ? row[fc[k]] : 0.0f;
       }
     }
 #pragma unroll
@@ -287,7 +287,7 @@ __device__ __forceinline__ void cand_cosines(const DivArgs& a, int b, int npool,
           const int cj = pk.c[min(c0 + lane + 32 * k, ncp - 1)];
 #pragma unroll
           for (int j = 0; j < kR; ++j)
-            if (e0 + j * step < npool) v[j][k] = __ldg(row[j] + cj);
+            if (e0 + j * step < npool) v[j][k] = row[j][cj];
         }
 #pragma unroll
         for (int j = 0; j < kR; ++j) {

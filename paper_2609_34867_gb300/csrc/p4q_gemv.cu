@@ -50,8 +50,8 @@ __device__ __forceinline__ int dp4a_us(uint32_t a, int b, int c) {
 
 template <int MR, bool S32>
 __global__ void __launch_bounds__(kGemvWarps * 32, kGemvCtas)
-    gemv_w4a4_kernel(const uint8_t* __restrict__ Xq, const float* __restrict__ s_a, int M, int K,
-                     const uint8_t* __restrict__ Wq, const float* __restrict__ s_w, int N, void* __restrict__ out) {
+    gemv_w4a4_kernel(const uint8_t* Xq, const float* s_a, int M, int K, const uint8_t* Wq, const float* s_w, int N,
+                     void* out) {
   extern __shared__ __align__(16) int8_t xs[];  // [M][K] sign-extended activation codes
   __shared__ int xsum[MR];                       // their row sums
   const int kb = K >> 1;                         // packed bytes per row

@@ -301,8 +301,8 @@ constexpr size_t kTokSmemThree = 72 * 1024;  // concept rows with three CTAs per
 
 template <int CH, int JMAX>
 __global__ void __launch_bounds__(256, kTokCtas)
-    select_token_quant_kernel(const uint16_t* __restrict__ V, int N, int L, int J, const uint8_t* __restrict__ qu,
-                              const int32_t* __restrict__ qsum, RowSinks out, float* __restrict__ qdots, int qp) {
+    select_token_quant_kernel(const uint16_t* V, int N, int L, int J, const uint8_t* qu, const int32_t* qsum,
+                              RowSinks out, float* qdots, int qp) {
   extern __shared__ __align__(16) uint8_t cq[];  // [J, L] the image's concept codes, expanded
   __shared__ uint32_t red_max[2][8];             // by row parity and warp
   __shared__ uint32_t red_sum[2][8][2 + JMAX];   // sums of u, of u^2 and of u u_j
@@ -529,7 +529,7 @@ constexpr int kRegMinRows = 2048;
 
 template <int CH, int G, bool NORM>
 __global__ void __launch_bounds__(256, 2)
-    quant_rows_reg_kernel(const uint16_t* __restrict__ X, long long ldx, int rows, int L, RowSinks out) {
+    quant_rows_reg_kernel(const uint16_t* X, long long ldx, int rows, int L, RowSinks out) {
   __shared__ uint32_t red[8][3];  // per warp: abs-max, sum of u, sum of u^2 (G > 1)
   pdl_wait();  // rows come from the previous kernel
   pdl_launch_dependents();

@@ -100,9 +100,8 @@ __device__ __forceinline__ float sum_to_f32(uint64_t lo, uint64_t hi) {
 
 template <int THREADS, int MAXC, bool EXPANDED>
 __global__ void __launch_bounds__(THREADS)
-    rmsnorm_quant_kernel(const __half* __restrict__ X, long long ldx, const __half* __restrict__ w, float eps, int K,
-                         uint8_t* __restrict__ Xq, float* __restrict__ s_a, uint8_t* __restrict__ Xu,
-                         int32_t* __restrict__ sum_xu) {
+    rmsnorm_quant_kernel(const __half* X, long long ldx, const __half* w, float eps, int K, uint8_t* Xq, float* s_a,
+                         uint8_t* Xu, int32_t* sum_xu) {
   pdl_launch_dependents();  // before the wait: see p4q_device.cuh
   pdl_wait();
   constexpr int kWarps = THREADS / 32;
@@ -117,7 +116,7 @@ __global__ void __launch_bounds__(THREADS)
 #pragma unroll
   for (int j = 0; j < MAXC; ++j) {
     const int c = t + j * THREADS;
-    xv[j] = c < nch ? __ldg(x4 + c) : make_uint4(0u, 0u, 0u, 0u);
+    xv[j] = c < nch ? x4[c] : make_uint4(0u, 0u, 0u, 0u);
   }
   // exact sum of squares
   uint32_t acc[4] = {0u, 0u, 0u, 0u};
@@ -154,7 +153,7 @@ __global__ void __launch_bounds__(THREADS)
 #pragma unroll
   for (int j = 0; j < MAXC; ++j) {
     const int c = t + j * THREADS;
-    const uint4 wv = c < nch ? __ldg(w4 + c) : make_uint4(0u, 0u, 0u, 0u);
+    const uint4 wv = c < nch ? w4[c] : make_uint4(0u, 0u, 0u, 0u);
     uint32_t xw[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
     const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll

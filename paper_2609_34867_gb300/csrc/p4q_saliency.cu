@@ -51,8 +51,8 @@ __device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_saddr) {
 // wph warps per head (a power of two); the CTA's heads in rounds of kWarps / wph.
 template <int DH, bool ONE>
 __global__ void __launch_bounds__(32 * kWarps, 2)
-    cls_saliency_kernel(const __half* __restrict__ q_cls, const __half* __restrict__ k_cls,
-                        const __half* __restrict__ k, int N, int C, int H, int cs_, int wph_, float* __restrict__ A) {
+    cls_saliency_kernel(const __half* q_cls, const __half* k_cls, const __half* k, int N, int C, int H, int cs_,
+                        int wph_, float* A) {
   // ONE: one CTA per crop, one warp per head
   const int cs = ONE ? 1 : cs_, wph = ONE ? 1 : wph_;
   pdl_wait();

@@ -56,10 +56,8 @@ constexpr int kSelThreads = 1024;
 // a hundred instructions, and every load of the scores goes out first.
 template <int PER>
 __global__ void __launch_bounds__(kSelThreads, 1)
-    select_stages12_kernel(const float* __restrict__ qdots, int qp, const int32_t* __restrict__ qnorm,
-                           const int32_t* __restrict__ vnorm, const float* __restrict__ A_cls, int N, int J, int Kq,
-                           int Ks, int Kd, uint32_t* __restrict__ kept12, int32_t* __restrict__ r0tok,
-                           int32_t* __restrict__ idx) {
+    select_stages12_kernel(const float* qdots, int qp, const int32_t* qnorm, const int32_t* vnorm, const float* A_cls,
+                           int N, int J, int Kq, int Ks, int Kd, uint32_t* kept12, int32_t* r0tok, int32_t* idx) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ RankScratch s;
@@ -138,8 +136,8 @@ __global__ void __launch_bounds__(kSelThreads, 1)
 // pool phase, that it does. Same layout and ranking as stages 1-2.
 template <int PER>
 __global__ void __launch_bounds__(kSelThreads, 1)
-    select_candidates_kernel(float* __restrict__ m, const float* __restrict__ mpart, int parts,
-                             const uint32_t* __restrict__ kept12, int N, int R0, int C, int32_t* __restrict__ cand) {
+    select_candidates_kernel(float* m, const float* mpart, int parts, const uint32_t* kept12, int N, int R0, int C,
+                             int32_t* cand) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ RankScratch s;
@@ -180,12 +178,9 @@ __global__ void __launch_bounds__(kSelThreads, 1)
 // ru[b, j] = vu[b, tok[b, j]] (d bytes), with its row sum and squared norm,
 // for R listed tokens per image (the kept set R0, or the candidates of the
 // diversity stage): one warp per row, 16-byte chunks.
-__global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t* __restrict__ vu,
-                                                          const int32_t* __restrict__ vsum,
-                                                          const int32_t* __restrict__ vnorm,
-                                                          const int32_t* __restrict__ tok, int B, int N, int d, int R,
-                                                          uint8_t* __restrict__ ru, int32_t* __restrict__ rsum,
-                                                          int32_t* __restrict__ rnorm) {
+__global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t* vu, const int32_t* vsum, const int32_t* vnorm,
+                                                          const int32_t* tok, int B, int N, int d, int R, uint8_t* ru,
+                                                          int32_t* rsum, int32_t* rnorm) {
   pdl_wait();
   pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
@@ -197,7 +192,10 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t* __restr
     const size_t src = static_cast<size_t>(b) * N + tok[r];
     const uint4* s = reinterpret_cast<const uint4*>(vu + src * d);
     uint4* t = reinterpret_cast<uint4*>(ru + static_cast<size_t>(r) * d);
-    for (int c = lane; c < chunks; c += 32) t[c] = ldg_stream16(s + c);
+    // (the token pass completed before this kernel was launched: the one in
+    // between let it launch after its own wait. 32 x 2880 tokens, whole call, us:
+    // 643 so, 654 with ordinary loads between the stores)
+    for (int c = lane; c < chunks; c += 32) t[c] = ldg_readonly16(s + c);
     if (lane == 0) {
       rsum[r] = vsum[src];
       rnorm[r] = vnorm[src];
@@ -217,11 +215,9 @@ constexpr int kCosmaxRows = 8;  // one row per warp: many warps in flight
 // cols == nullptr: column j of a row is R0 token j (the R0 GEMM's output,
 // norms r0norm); else the row holds every token (the Gram mode's cdots) and
 // column j is token cols[b, j] (norms from vnorm).
-__global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* __restrict__ dots, int pitch,
-                                                        const int32_t* __restrict__ vnorm,
-                                                        const int32_t* __restrict__ r0norm,
-                                                        const int32_t* __restrict__ cols, int N, int R0,
-                                                        float* __restrict__ m) {
+__global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* dots, int pitch, const int32_t* vnorm,
+                                                        const int32_t* r0norm, const int32_t* cols, int N, int R0,
+                                                        float* m) {
   extern __shared__ int32_t nr[];  // [R0] squared norms of the image's kept tokens, [R0] their rsqrtf, [R0] columns
   float* rr = reinterpret_cast<float*>(nr + R0);
   int32_t* cj = nr + 2 * R0;
@@ -243,13 +239,13 @@ __global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* __restrict_
     const float ra = na > 0 ? rsqrtf(static_cast<float>(na)) : 0.0f;
     float amax = -INFINITY;
 #pragma unroll 4
-    for (int j = lane; j < R0; j += 32) amax = fmaxf(amax, __ldg(dr + cj[j]) * ra * rr[j]);
+    for (int j = lane; j < R0; j += 32) amax = fmaxf(amax, dr[cj[j]] * ra * rr[j]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
     float emax = -INFINITY;
 #pragma unroll 4
     for (int j = lane; j < R0; j += 32) {
-      const float dot = __ldg(dr + cj[j]);
+      const float dot = dr[cj[j]];
       if (dot * ra * rr[j] >= amax - kCosMargin) emax = fmaxf(emax, code_cosine(static_cast<int>(dot), na, nr[j]));
     }
 #pragma unroll
@@ -267,8 +263,7 @@ __global__ void __launch_bounds__(256) r0_cosmax_kernel(const float* __restrict_
 __device__ __forceinline__ uint32_t score_key(float v) { return float_order_key(v == 0.0f ? 0.0f : v); }
 
 __global__ void __launch_bounds__(kSelThreads)
-    topk_replacement_kernel(const float* __restrict__ s_ref, const float* __restrict__ s_alt, int N, int K,
-                            int32_t* __restrict__ inter, float* __restrict__ rho) {
+    topk_replacement_kernel(const float* s_ref, const float* s_alt, int N, int K, int32_t* inter, float* rho) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ RankScratch s;

@@ -118,9 +118,8 @@ __device__ __forceinline__ void swiglu8(const uint32_t (&ng)[4], const uint32_t 
 
 template <int THREADS, int MAXC, bool EXPANDED>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (MAXC <= 3 ? 4 : 2) : THREADS == 384 ? 3 : 2)
-    swiglu_quant_kernel(const __half* __restrict__ gate, long long ldg, const __half* __restrict__ up, long long ldu,
-                        int K, uint8_t* __restrict__ Xq, float* __restrict__ s_a, uint8_t* __restrict__ Xu,
-                        int32_t* __restrict__ sum_xu) {
+    swiglu_quant_kernel(const __half* gate, long long ldg, const __half* up, long long ldu, int K, uint8_t* Xq,
+                        float* s_a, uint8_t* Xu, int32_t* sum_xu) {
   pdl_launch_dependents();  // before the wait: see p4q_device.cuh
   pdl_wait();
   __shared__ float wmax[THREADS / 32];
