@@ -4,8 +4,8 @@
 // is empty); each of the K_d rounds keeps the free token with the smallest
 // m (lower index on ties) and m absorbs its cosines.
 //
-// One CTA per image (and, up to 32 images, three helpers that share phase 2's
-// cosines). The largest cosine of every token to R0 comes from the
+// One CTA per image (and, while that leaves SMs free, one or three helpers that
+// share phase 2's cosines). The largest cosine of every token to R0 comes from the
 // tensor-core GEMM before this kernel (its cosine-max epilogue, or a row pass
 // over its int32 tiles; in Gram mode a row pass over the token-pair GEMM)
 // as m. After that no cosine row of the whole image is ever formed. The kernel holds, for every free token, a
@@ -738,11 +738,17 @@ cudaError_t launch_select_diverse(const SelectPlan& p, const SelectWorkspace& ws
   a.K = p.K;
   a.Kd = p.Kd;
   a.idx = idx;
-  // Four CTAs per image while their clusters surely run side by side (128 of
-  // the 152 SMs; a cluster's CTAs are of one SM group). Whole selector call, us,
-  // clusters of 1 / 4 / 8: 1 x 576 tokens 47.3 / 45.7 / 45.6, 16 x 576 110.3 /
-  // 109.7 / 120.2, 32 x 2880 765 / 753 / 832.
-  const int cs = p.B <= 32 ? 4 : 1;
+  // Each CTA takes an SM, most of whose time a helper waits: so as many per image
+  // as leave room for another selection's on a second stream. Four while two
+  // calls' take half the SMs (9 images of 152 SMs), two while they fit (38).
+  // Whole selector call of 576 tokens (K = 192) / 2880 tokens (K = 640), us,
+  // clusters of 1, 2, 4:
+  //   one stream: 1 image 66.4 -> 63.4, 60.7 / 458 -> 454, 449; 8 images 89.0 ->
+  //     86.7, 83.0 / 675 -> 671, 664; 32 images 162 -> 159, 156 / 1002 -> 994, 990;
+  //   two streams, per call: 8 images 57.0 -> 55.6, 55.7 / 374 -> 371, 372; 12
+  //     64.9 -> 62.5, 70.2 / 430 -> 427, 429; 16 86.0 -> 85.9, 89.6 / 489 -> 488,
+  //     517; 32 141 -> 130, 137 / 705 -> 718, 833.
+  const int sms = num_sms(), cs = 16 * p.B <= sms ? 4 : 4 * p.B <= sms ? 2 : 1;
   auto go = [&](auto kern, int threads) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDivSmem));
     if (e != cudaSuccess) return e;

@@ -261,9 +261,9 @@ def test_diversity_block_widths(p4q, dev, N, K):
     assert np.array_equal(idx.cpu().numpy(), oracle.select_batch(x.V, K, x.Q, x.A))
 
 
-@pytest.mark.parametrize("B", [32, 33])
+@pytest.mark.parametrize("B", [9, 10, 32, 33, 38, 39])
 def test_diversity_image_counts(p4q, dev, B):
-    """Stage 3 with and without helper CTAs (clusters up to 32 images)."""
+    """Stage 3 with three, one and no helper CTAs per image (152 SMs: up to 9, 38 and more images)."""
     w = wl.Workload("t", B=B, N=300, d=128, K=200, T=0, J=2, seed=B, heavy_tail=False, linears=())
     x = wl.selector_inputs(w)
     idx = p4q.select(torch.from_numpy(x.V).to(dev), torch.from_numpy(x.Q).to(dev), torch.from_numpy(x.A).to(dev), w.K)
