@@ -56,7 +56,7 @@ constexpr uint32_t kTmemCols = 256;
 
 struct DivScratch {
   RankScratch rank;
-  int t, npool, tmin, nphase;
+  int t, npool, tmin;
   unsigned long long tau;
   __align__(16) uint32_t skey[kPool];   // pool rounds: order keys of the certain entries' m
   int prank[kPool];                     // pool rounds: their ranks
@@ -375,7 +375,6 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
     mbar_init(&s.bar_done, 1);
     s.abort_flag = 0;
     s.t = 0;
-    s.nphase = 0;
     fence_barrier_init();
   }
   if (warp == 0) {
@@ -414,13 +413,16 @@ __global__ void __launch_bounds__(kThreads, 1) select_diverse_kernel(const DivAr
   int chunks = 0;  // accumulators completed so far (phases of bar_acc)
   uint32_t key[PER];
 
-  while (true) {
+  // Every thread leaves the loop at the same phase: what it decides on changes
+  // only behind a later barrier of the block (s.t; the abort flag of the bounded
+  // waits), or is its own count of the phases.
+  for (int phase = 0;; ++phase) {
     __syncthreads();
     const int t = s.t;
     if (t >= a.Kd || s.abort_flag) break;
-    if (threadIdx.x == 0 && ++s.nphase > phase_limit) {
-      s.abort_flag = 1;
-      atomicOr(&g_diverse_err, kErrTimeout);
+    if (phase >= phase_limit) {
+      if (threadIdx.x == 0) atomicOr(&g_diverse_err, kErrTimeout);
+      break;
     }
 #pragma unroll
     for (int e = 0; e < PER; ++e)
