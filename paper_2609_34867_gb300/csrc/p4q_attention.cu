@@ -658,13 +658,9 @@ cudaError_t launch_causal_attention(const uint16_t* q, long long ldq, const uint
                                     const uint16_t* v, long long ldv, int B, int m, int H, int Hkv, uint16_t* o,
                                     long long ldo, cudaStream_t stream) {
   if (B <= 0) return cudaSuccess;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(causal_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(causal_attention_kernel, kSmemBytes);
+  if (le != cudaSuccess) return le;
   CUtensorMap mq, mk, mv, mo;
   if (!make_rows_map(&mq, q, B, m, H * kDH, ldq, 128)) return cudaErrorInvalidValue;
   if (!make_rows_map(&mk, k, B, m, Hkv * kDH, ldk, 128)) return cudaErrorInvalidValue;

@@ -452,13 +452,9 @@ bool make_packed_map(CUtensorMap* map, const uint8_t* base, int K, int rows) {
 
 template <bool S32>
 cudaError_t launch_out(const GemmArgs& g, cudaStream_t stream) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(w4a4_fewrows_kernel<S32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(w4a4_fewrows_kernel<S32>, kSmemMax);
+  if (le != cudaSuccess) return le;
   const int KB = g.K / kBK;
   FewParams p;
   p.X = g.A;

@@ -994,13 +994,9 @@ namespace {
 template <int BN, int MODE>
 cudaError_t launch_cfg(const GemmArgs& g, cudaStream_t stream) {
   using C = Cfg<BN, MODE>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(w4a4_gemm_kernel<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(w4a4_gemm_kernel<BN, MODE>, C::SMEM);
+  if (le != cudaSuccess) return le;
   CUtensorMap ma, mb, md;
   if (!make_operand_map(&ma, g.A, g.K, g.M, g.batch, g.a_batch_stride, BM)) return cudaErrorInvalidValue;
   if (!make_operand_map(&mb, g.B, g.K, g.N, g.batch, g.b_batch_stride, BN)) return cudaErrorInvalidValue;
@@ -1028,13 +1024,9 @@ cudaError_t launch_cfg(const GemmArgs& g, cudaStream_t stream) {
 
 template <int MODE>
 cudaError_t launch_pair(const GemmArgs& g, cudaStream_t stream) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(pair::w4a4_gemm_pair_kernel<MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, pair::Lay<MODE>::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(pair::w4a4_gemm_pair_kernel<MODE>, pair::Lay<MODE>::SMEM);
+  if (le != cudaSuccess) return le;
   CUtensorMap ma, mb, md;
   if (!make_operand_map(&ma, g.A, g.K, g.M, g.batch, g.a_batch_stride, BM)) return cudaErrorInvalidValue;
   if (!make_operand_map(&mb, g.B, g.K, g.N, g.batch, g.b_batch_stride, pair::HB)) return cudaErrorInvalidValue;

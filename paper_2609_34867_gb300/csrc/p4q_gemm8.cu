@@ -514,13 +514,9 @@ cudaError_t launch8(const GemmArgs& g, const Ws8& w, cudaStream_t stream) {
   const int bn = (MODE != static_cast<int>(GemmOut::kHalf)) ? g.tile_n : BN;
   if (bn < 32 || bn > BN || bn % 32 != 0) return cudaErrorInvalidValue;
   if (MODE == kCosMode && (!g.norm_a || !g.norm_b || !g.D)) return cudaErrorInvalidValue;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(w4a4_gemm8_pair_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Lay8<MODE>::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(w4a4_gemm8_pair_kernel<MODE>, Lay8<MODE>::SMEM);
+  if (le != cudaSuccess) return le;
   CUtensorMap ma, mb, md;
   const int batch = g.batch > 0 ? g.batch : 1;
   if (!make_expanded_map(&ma, w.a8, g.K, g.M, batch, BM)) return cudaErrorInvalidValue;

@@ -172,13 +172,9 @@ __global__ void __launch_bounds__(kGemvWarps * 32, kGemvCtas)
 template <int MR, bool S32>
 cudaError_t launch_mr(const GemmArgs& g, cudaStream_t stream) {
   const size_t smem = static_cast<size_t>(g.M) * g.K;
-  static size_t smem_set = 48u << 10;
-  if (smem > smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemv_w4a4_kernel<MR, S32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kGemvSmemMax));
-    if (e != cudaSuccess) return e;
-    smem_set = kGemvSmemMax;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(gemv_w4a4_kernel<MR, S32>, kGemvSmemMax);
+  if (le != cudaSuccess) return le;
   // enough warps for every pair of weight rows, at most the CTAs that fit on the SMs
   const int per_sm = smem <= 64u * 1024u ? kGemvCtas : smem <= 100u * 1024u ? 2 : 1;
   const int want = (g.N / 2 + kGemvWarps - 1) / kGemvWarps;

@@ -9,6 +9,8 @@
 
 #include <utility>
 
+#include "p4q_smem_limit.h"
+
 namespace p4q {
 
 // Launches kernel<<<grid, block, smem, stream>>>(args...) with programmatic

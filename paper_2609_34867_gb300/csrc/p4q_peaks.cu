@@ -161,13 +161,10 @@ size_t peak_probe_sink_words() { return 8 * 1024; }
 cudaError_t launch_peak_probe(int kind, int iters, uint32_t* sink, double* ops, cudaStream_t stream) {
   const int sms = num_sms();
   if (kind == 0) {
-    static bool attr_set = false;
+    static SmemLimit limit;
     const int smem = 1024 + 2 * kTcTileBytes + 64;
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(tc_peak_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      attr_set = true;
-    }
+    const cudaError_t le = limit.allow(tc_peak_kernel, smem);
+    if (le != cudaSuccess) return le;
     const int ctas = 2 * (sms / 2);
     *ops = 2.0 * 256 * 256 * 32 * 4.0 * iters * (ctas / 2);
     return launch_pdl(tc_peak_kernel, dim3(ctas), dim3(kTcThreads), smem, stream, iters, sink);

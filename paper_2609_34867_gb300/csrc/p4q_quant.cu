@@ -250,13 +250,9 @@ int sm_count() {
 template <int G, bool NORM>
 cudaError_t launch_g(const RowSource& src, int rows, int L, const RowSinks& out, const RowSinks& out2, const Plan& p,
                      cudaStream_t stream) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(quant_rows_kernel<G, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSmemMax);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(quant_rows_kernel<G, NORM>, kSmemMax);
+  if (le != cudaSuccess) return le;
   constexpr int kGroups = kWarps / G;
   const size_t smem = static_cast<size_t>(kGroups) * p.S * p.stage_bytes + kGroups * kMaxStages * 8 +
                       3 * kWarps * 4 + kGroups * 4;
@@ -418,13 +414,9 @@ template <int CH, int JMAX>
 cudaError_t launch_token_quant(const uint16_t* V, int B, int N, int L, int J, const uint8_t* qu, const int32_t* qsum,
                                const RowSinks& out, float* qdots, int qp, cudaStream_t stream) {
   const size_t smem = static_cast<size_t>(J) * L;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(select_token_quant_kernel<CH, JMAX>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t le = limit.allow(select_token_quant_kernel<CH, JMAX>, 100 * 1024);
+  if (le != cudaSuccess) return le;
   // at most as many CTAs as run at once over the whole batch (one wave: rows are dealt out per CTA in
   // advance, so a second wave would double the time), never more pairs of warps than an image has rows
   const int ctas = smem <= kTokSmemThree ? kTokCtas : 2;

@@ -31,6 +31,7 @@ namespace {
 constexpr int kWarps = 16;
 constexpr int kMaxHeads = 32;
 constexpr int kMaxCluster = 8;
+constexpr size_t kSmemMax = 227u * 1024u - 256u;  // dynamic, beside the reductions
 
 // Lanes that share one token's key row: the row's dh / 8 16-byte chunks, one
 // per lane, rounded up to a power of two (idle lanes past the row).
@@ -197,20 +198,16 @@ cudaError_t launch_dh(const __half* q_cls, const __half* k_cls, const __half* k,
   int cs = 1;
   auto weights = [&](int x) { return static_cast<size_t>((H + x - 1) / x) * (N / C) * sizeof(float); };
   while (cs < kMaxCluster && 2 * cs <= H &&
-         (static_cast<long long>(B) * C * 2 * cs <= 2 * num_sms() || weights(cs) + 256 > 227u * 1024u))
+         (static_cast<long long>(B) * C * 2 * cs <= 2 * num_sms() || weights(cs) > kSmemMax))
     cs *= 2;
   const int heads = (H + cs - 1) / cs;
   int wph = 1;  // warps per head: the CTA's warps over its heads
   while (2 * wph * heads <= kWarps) wph *= 2;
   const size_t smem = weights(cs);
-  static size_t smem_set = 48u << 10;
-  if (smem > smem_set) {
-    for (auto kern : {cls_saliency_kernel<DH, true>, cls_saliency_kernel<DH, false>}) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-      if (e != cudaSuccess) return e;
-    }
-    smem_set = smem;
-  }
+  static SmemLimit limit_one, limit_more;
+  const cudaError_t le = cs == 1 && wph == 1 ? limit_one.allow(cls_saliency_kernel<DH, true>, kSmemMax)
+                                             : limit_more.allow(cls_saliency_kernel<DH, false>, kSmemMax);
+  if (le != cudaSuccess) return le;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(C) * cs, B);
   cfg.blockDim = dim3(32 * kWarps);
