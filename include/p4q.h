@@ -85,13 +85,15 @@ uint64_t p4q_launch_count(void);
 
 /* GEMM kernel variant used by p4q_w4a4_linear and p4q_w4a4_gemm_s32, for all
  * later calls in the process (for tests and tuning; results are identical):
- *   0 automatic (default): for M <= 2 rows a weight-streaming kernel (dp4a
- *     on the CUDA cores: the packed weights are read once); for few rows (M
- *     <= 128 and M * ceil(N / 128) <= 8192) a kernel with the weights on the
- *     tensor cores' row side and k split over a cluster; CTA-pair kernel for
- *     fp16 outputs with M >= 256 and N >= 256, or with N >= 1024 from M = 129
- *     (from M = 65 while ceil(N / 256) <= the CTA pairs of the GPU);
- *     single-CTA kernel otherwise;
+ *   0 automatic (default): for M <= 2 rows, and up to 8 on small weights, a
+ *     weight-streaming kernel (dp4a on the CUDA cores: the packed weights are
+ *     read once); for up to 128 rows, fewer for more weight rows and for Kin <
+ *     1024 or > 8192, a kernel with the weights on the tensor cores' row side and
+ *     k split over a cluster; CTA-pair kernel for fp16 outputs with M >= 256
+ *     and N >= 256, or with N >= 1024 and Kin >= 2048 from M = 129 (from M = 65
+ *     while ceil(N / 256) <= the CTA pairs of the GPU); single-CTA kernel
+ *     otherwise (where each line lies: p4q_gemv.cu, p4q_fewrows.cu,
+ *     p4q_gemm.cu);
  *   1 single-CTA kernel only;
  *   2 CTA-pair kernel whenever N >= 256 (also for int32 outputs);
  *   3 like 0, and the workspace entry points take the expanded-operand path

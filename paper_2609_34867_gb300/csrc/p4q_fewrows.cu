@@ -522,14 +522,26 @@ cudaError_t launch_out(const GemmArgs& g, cudaStream_t stream) {
 // memory: a second tile reads the weights again, against that file's CTA pairs
 // (128 x 5120 x 5120 27.9 / 29.3, 96 x 5120 x 13824 45.3 / 62.2, 128 x 4096 x
 // 11008 56.2 / 51.5, 128 x 5120 x 13824 74.6 / 62.2).
+// Its int32 outputs have no pairs there: a second tile while the CTAs are at most
+// three rounds (128 x 2048 x 11008 32.3 / 50.9, 128 x 5120 x 8320 59.1 / 40.0).
+// Short rows: the unpacking, sums and outputs of a row tile cost this kernel more
+// per row than that file's, whose time is that of its k loop (64 x 256 x 128 8.1 /
+// 5.4, 32 x 256 x 256 5.6 / 6.0, 48 x 256 x 256 6.7 / 6.0, 64 x 256 x 512 6.3 / 7.0, 96 x
+// 256 x 512 7.8 / 7.0; fp16 outputs from N = 1024, where that file takes wider tiles:
+// 48 x 1024 x 128 7.2 / 7.4, 64 x 1024 x 256 7.6 / 8.3, 80 x 1024 x 256 8.9 / 8.4, 96 x 1024 x
+// 512 8.0 / 9.7).
 bool fewrows_applies(const GemmArgs& g) {
   const int nkb = (g.K / kBK + kMaxCluster - 1) / kMaxCluster;
   const bool one_tile = g.M <= kMaxRowTile && 1024 + few_x_bytes(g.M, (g.M + 16) / 16 * 16, (g.M + 8) / 8 * 8, nkb) +
                                                       2 * kPairBytes <= kSmemMax;
   const bool pairs_serve = g.out == GemmOut::kHalf && g.N >= 1024 && (g.N + 255) / 256 <= num_sms() / 2;
+  const long long ntiles = (g.N + kTileN - 1) / kTileN;
+  const bool second_tile = g.out == GemmOut::kHalf ? !pairs_serve : 2 * kMaxCluster * ntiles <= 3 * num_sms();
+  const int mt = g.M <= kMaxRowTile ? g.M : (g.M + 1) / 2;
+  const int rows = std::max(24, g.K / 8) + (g.out == GemmOut::kHalf && g.N >= 1024 ? 32 : 0);
   return (g.out == GemmOut::kHalf || g.out == GemmOut::kS32) && g.batch == 1 && g.M >= 1 && g.M <= 128 &&
-         static_cast<long long>(g.M) * ((g.N + kTileN - 1) / kTileN) <= 8192 && g.N % 2 == 0 && g.K % kBK == 0 &&
-         (g.d_pitch == 0 || g.d_pitch == g.N) && (g.K <= 8192 || one_tile || !pairs_serve);
+         g.M * ntiles <= (g.K >= 512 ? 8192 : 6144) && (g.K >= 1024 || mt <= rows) && g.N % 2 == 0 && g.K % kBK == 0 &&
+         (g.d_pitch == 0 || g.d_pitch == g.N) && (g.K <= 8192 || one_tile || second_tile);
 }
 
 cudaError_t launch_fewrows(const GemmArgs& g, cudaStream_t stream) {

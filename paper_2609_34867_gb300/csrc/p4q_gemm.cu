@@ -1071,8 +1071,11 @@ cudaError_t launch_w4a4_gemm(const GemmArgs& g, cudaStream_t stream) {
   // run one round where the pairs need two). Measured (us, single / pair): 160 x
   // 256 x 4096 (N x K) 21.7 / 24.6, 160 x 1024 x 4096 29.0 / 25.0, 160 x 4096 x
   // 11008 71.1 / 51.5, 160 x 27648 x 5120 73.3 / 52.6, 96 x 12288 x 4096 29.7 /
-  // 25.9, 96 x 22016 x 4096 30.6 / 43.7, 33 x 12288 x 4096 33.4 / 42.5.
-  const bool pair_rows = g.M >= 256 || (g.N >= 1024 && (g.M > 128 || (g.M > 64 && (g.N + 255) / 256 <= num_sms() / 2)));
+  // 25.9, 96 x 22016 x 4096 30.6 / 43.7, 33 x 12288 x 4096 33.4 / 42.5. Below K =
+  // 2048 the pairs' longer start is not made up for: 192 x 4096 x 512 9.9 / 11.4, x
+  // 1024 12.8 / 13.7, x 1536 15.6 / 15.7, x 2048 18.3 / 17.6.
+  const bool pair_rows =
+      g.M >= 256 || (g.N >= 1024 && g.K >= 2048 && (g.M > 128 || (g.M > 64 && (g.N + 255) / 256 <= num_sms() / 2)));
   const bool pair_ok = g.M > 0 && g.N >= 256 && g.batch > 0 && g_pair_mode != 0 &&
                        (g_pair_mode == 1 || (pair_rows && g.out == GemmOut::kHalf));
   if (pair_ok && g.out == GemmOut::kHalf) return launch_pair<0>(g, stream);

@@ -44,3 +44,12 @@ def test_fewrows_bit_exact(p4q, dev, M, N, K):
 def test_dispatch_edges(p4q, dev, M, N, K):
     """Around the lines between the few-rows kernel, the CTA pairs and the single CTAs."""
     test_fewrows_bit_exact(p4q, dev, M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(24, 256, 128), (25, 256, 128), (56, 1024, 128), (57, 1024, 128), (64, 1024, 256),
+                                   (65, 1024, 256), (127, 1032, 512), (128, 1032, 512), (96, 264, 768), (97, 264, 768),
+                                   (48, 16384, 384), (49, 16384, 384), (128, 3640, 8320), (128, 3656, 8320),
+                                   (192, 1024, 1920), (192, 1024, 2048)])
+def test_dispatch_edges_of_short_rows(p4q, dev, M, N, K):
+    """Around the lines that Kin moves, for fp16 and int32 outputs."""
+    test_fewrows_bit_exact(p4q, dev, M, N, K)
