@@ -4,20 +4,20 @@
 // crop's patch keys, of q . k / sqrt(d_h), and the saliency of a patch is its
 // weight averaged over the heads.
 //
-// Kernel: a cluster of up to 8 CTAs per (image, crop), its heads dealt out to
-// the CTAs and each head's tokens to the CTA's warps, so that a few crops
-// still occupy many SMs. A token's key row for the head (dh fp16 values, rows
-// of consecutive tokens H x dh apart) is read by dh / 8 lanes with one 16-byte
-// load each, so that a warp load covers whole rows; the lanes' partial dot
-// products (fp16 products accumulated in fp32) are summed by shuffles. The
-// head's max and sum (over its warps, in warp order) give its softmax; the
-// per-head weights stay in the CTA's shared memory, and each CTA sums its share
-// of the tokens over the heads in head order, reading the other CTAs' weights
-// through distributed shared memory (deterministic for a given shape).
+// Kernel: one CTA per (image, crop) or, where that leaves SMs idle, a cluster of
+// up to 8, its heads dealt out to the CTAs and each head's tokens to the CTA's
+// warps. A token's key row for the head (dh fp16 values, rows of consecutive
+// tokens H x dh apart) is read by dh / 8 lanes with one 16-byte load each, so
+// that a warp load covers whole rows; the lanes' partial dot products (fp16
+// products accumulated in fp32) are summed by shuffles. The head's max and sum
+// (over its warps, in warp order) give its softmax; the per-head weights stay in
+// the CTA's shared memory, and each CTA sums its share of the tokens over the
+// heads in head order, reading the other CTAs' weights through distributed
+// shared memory (deterministic for a given shape).
 //
 // Bound: load latency for few crops, HBM for many. Measured (16 heads x 64, us;
 // one CTA per crop and one warp per head before): 8 crops of 576 tokens 8.2
-// (24.3), 32 crops 13.7 (31.9), 80 crops 30.2 (34.4), 160 crops 44.5 (46.9) =
+// (24.3), 32 crops 13.7 (31.9), 80 crops 29.1 (29.9), 160 crops 44.3 (47.4) =
 // 4.2 TB/s, 4 crops of 3600 at 128 wide 66 (390).
 #include <cuda_fp16.h>
 
@@ -49,7 +49,7 @@ __device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_saddr) {
   return v;
 }
 
-// wph warps per head (a power of two); the CTA's heads in rounds of kWarps / wph.
+// wph warps per head (a power of two); the CTA's heads in rounds of its warps / wph.
 template <int DH, bool ONE>
 __global__ void __launch_bounds__(32 * kWarps, 2)
     cls_saliency_kernel(const __half* q_cls, const __half* k_cls, const __half* k, int N, int C, int H, int cs_,
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = lane % LPT, tok = lane / LPT;
   const int mine = heads_of(H, cs, rank);
-  const int hpr = kWarps / wph;              // heads per round
+  const int hpr = static_cast<int>(blockDim.x >> 5) / wph;  // heads per round
   const int part = warp % wph;               // this warp's part of the head's tokens
   const int per = (n + wph - 1) / wph, t0 = part * per, t1 = min(n, t0 + per);
   const float scale = 1.0f / sqrtf(static_cast<float>(DH));
@@ -193,16 +193,34 @@ __global__ void __launch_bounds__(32 * kWarps, 2)
 template <int DH>
 cudaError_t launch_dh(const __half* q_cls, const __half* k_cls, const __half* k, int B, int N, int C, int H,
                       float* A, cudaStream_t stream) {
-  // CTAs per crop: as many as leave every SM at most two, and one head each;
-  // more where one CTA's weights and its reductions exceed the shared memory
+  // CTAs per crop. A cluster pays where a crop's keys are some work for a CTA and
+  // SMs are free: from 80 KB of keys (twice that when every SM has a crop), as many
+  // CTAs as one per SM, or two per SM from 1 MB. Elsewhere one CTA, a warp per
+  // head, is faster: 16 heads x 64, us, clusters of up to two CTAs per SM always /
+  // this: 8 crops of 49 tokens 4.8 / 4.4, 75 of 49 9.0 / 4.6, 75 of 196 14.4 / 9.5, 100
+  // of 400 22.1 / 16.7, 40 of 576 16.8 / 16.6. More CTAs where one's weights exceed
+  // its shared memory.
+  const long long crops = static_cast<long long>(B) * C, sms = num_sms();
+  const long long keys = 2ll * H * (N / C) * DH;  // bytes
   int cs = 1;
   auto weights = [&](int x) { return static_cast<size_t>((H + x - 1) / x) * (N / C) * sizeof(float); };
-  while (cs < kMaxCluster && 2 * cs <= H &&
-         (static_cast<long long>(B) * C * 2 * cs <= 2 * num_sms() || weights(cs) > kSmemMax))
-    cs *= 2;
-  const int heads = (H + cs - 1) / cs;
-  int wph = 1;  // warps per head: the CTA's warps over its heads
-  while (2 * wph * heads <= kWarps) wph *= 2;
+  auto split = [&](int x) {
+    return weights(x) > kSmemMax || (keys * sms >= 80 * 1024 * (sms + crops) &&
+                                     crops * 2 * x <= (keys >= 1 << 20 ? 2 * sms : sms));
+  };
+  while (cs < kMaxCluster && 2 * cs <= H && split(cs)) cs *= 2;
+  // Warps per head. In a cluster, all of the block's; one CTA's, several where the
+  // head's tokens are many rounds of loads and the SMs have room (16 warps each,
+  // 32 for long crops): 400 crops of 49 tokens, 4 heads x 64, two / one 7.2 / 4.3.
+  const int heads = (H + cs - 1) / cs, n = N / C;
+  constexpr int kTokens = 32 / lanes_per_token<DH>();  // per warp and load
+  int wph = 1;
+  auto share = [&](int x) {
+    const long long warps = crops * heads * x * 2;
+    return cs > 1 || (warps <= 16 * sms && n > 12 * x * kTokens) || (warps <= 32 * sms && n > 64 * x * kTokens);
+  };
+  while (2 * wph * heads <= kWarps && share(wph)) wph *= 2;
+  const int warps = heads * wph < kWarps ? heads * wph : kWarps;
   const size_t smem = weights(cs);
   static SmemLimit limit_one, limit_more;
   const cudaError_t le = cs == 1 && wph == 1 ? limit_one.allow(cls_saliency_kernel<DH, true>, kSmemMax)
@@ -210,7 +228,7 @@ cudaError_t launch_dh(const __half* q_cls, const __half* k_cls, const __half* k,
   if (le != cudaSuccess) return le;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(C) * cs, B);
-  cfg.blockDim = dim3(32 * kWarps);
+  cfg.blockDim = dim3(32 * warps);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];

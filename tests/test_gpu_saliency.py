@@ -68,10 +68,20 @@ def test_saliency_feeds_the_selector(p4q, dev):
                                         (80, 1, 25, 16, 64), (160, 1, 20, 16, 64), (90, 2, 9, 5, 128),
                                         (1, 1, 3632, 16, 32), (200, 1, 3, 1, 64)])
 def test_saliency_clusters(p4q, dev, B, C, n, H, dh):
-    """Heads over clusters of 8, 4, 2 and 1 CTAs (evenly or not), one or
-    several warps per head, the largest weights one CTA was asked to hold."""
+    """Small crops (one CTA each), a cluster for a long one, the largest
+    weights one CTA was asked to hold."""
     rng = np.random.default_rng(B + n + H)
     q = (rng.standard_normal((B, C, H, dh)) * 2).astype(np.float16)
     kc = rng.standard_normal((B, C, H, dh)).astype(np.float16)
     k = rng.standard_normal((B, C * n, H, dh)).astype(np.float16)
     _check(p4q, dev, q, kc, k)
+
+
+@pytest.mark.parametrize("B,C,n,H,dh", [(1, 3, 200, 12, 64), (19, 1, 120, 16, 64), (20, 1, 120, 16, 64), (5, 5, 200, 7, 80),
+                                        (38, 1, 190, 6, 128), (39, 2, 100, 16, 64), (38, 2, 150, 16, 64),
+                                        (77, 1, 520, 16, 64), (80, 1, 600, 4, 32), (152, 1, 300, 3, 64),
+                                        (300, 1, 600, 4, 32), (10, 1, 42, 16, 64), (2, 1, 45, 30, 32)])
+def test_saliency_splits(p4q, dev, B, C, n, H, dh):
+    """Clusters of 8, 4 and 2 CTAs and none on either side of the lines between
+    them, heads that divide evenly or not, one CTA with several warps per head."""
+    test_saliency_clusters(p4q, dev, B, C, n, H, dh)
