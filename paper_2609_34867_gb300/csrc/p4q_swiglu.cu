@@ -1,30 +1,31 @@
 // SwiGLU before down_proj, fused with the per-token 4-bit quantizer of
 // down_proj's input (App. A: every linear's input is quantized per token):
 //   h = silu(gate) * up, silu(g) = g * (1 / (1 + exp32(-g))) (each
-//   operation one rounded fp32 step, the reciprocal within 0.51 ulp),
+//   operation one rounded fp32 step, the reciprocal correctly rounded),
 //   then a = max|h|, s = a / 7, code = clamp(round_half_even(h / s), -8, 7).
 // exp32 is an own fp32 exponential (Cody-Waite reduction with ln 2 split as
 // 355/512 + a low part, degree-7 Taylor polynomial by Horner's rule with fused
 // multiply-adds, two exact power-of-two scalings; within 0.9 ulp of e^x; 0
-// below -87, inf above 88.72284). The fp32 h is within 2.91 ulp (3.5e-7
-// relative: 0.9 ulp from exp32, three roundings of 2^-24 and the reciprocal's
-// 0.51 ulp) of the real
+// below -87, inf above 88.72284). The fp32 h is within 2.9 ulp (3.5e-7
+// relative: 0.9 ulp from exp32 and four roundings of 2^-24) of the real
 // silu(g) * up, the row's abs-max likewise, the scale a / 7 adds one
 // rounding and the quotient h / s one more, so h / s is within 8.1e-7
 // relative, 5.7e-6 absolute (|h / s| <= 7), of the exact quotient: the codes
 // are those of the exact SwiGLU except where that quotient falls within
 // 5.7e-6 of a .5 boundary.
 //
-// Kernel: one CTA per row (256, 384 or 512 threads); each thread holds its chunks of 8 values of h in registers
-// (computed once), the row's abs-max comes from a block reduction, then the
-// codes are written packed and, optionally, expanded one byte per code (u =
+// Kernel: one CTA per row (256, 384 or 512 threads); each thread holds its
+// chunks of 8 values of h in registers (computed once), the row's abs-max comes
+// from a block reduction, then the codes are written packed and, optionally, expanded one byte per code (u =
 // code + 8, the GEMM's order) with their row sum.
 //
 // Bound: instruction issue, then HBM. Gates within [-87, 87] (nearly all
 // chunks; the others take the scalar form below) are evaluated two at a time
 // (fma.rn.f32x2), the power of two enters the exponent by an integer addition,
 // the reciprocal is the hardware approximation with one Newton step (Markstein's
-// correction: residual by a fused multiply-add), and the codes come from
+// correction: residual by a fused multiply-add; compared with the correctly
+// rounded reciprocal for every significand at the exponents 0 .. 125, which hold
+// 1 + e^87: equal, so that both forms give the same h), and the codes come from
 // the bracketing products of p4q_codes.cuh: about 20 instructions per value
 // where one at a time with a library reciprocal took about 45. Measured (us,
 // inputs past L2; before): 6144 x 11008 84 (140) = 4.4 TB/s, 6144 x 13824 104

@@ -109,3 +109,25 @@ def test_swiglu_quant_widths(p4q, dev, M, K):
     at = rng.integers(0, K, M)
     g[np.arange(M), at] = rng.choice(np.array([-500.0, -90.0, -88.0, -87.0, 87.0, 87.06, 88.0, 300.0]), M)
     _check(p4q, dev, g, u)
+
+
+def test_both_forms_give_the_same_h(p4q, dev):
+    """Every finite fp16 gate, evaluated with its chunk two values at a time and,
+    where another gate of the chunk lies past 87, one at a time (correctly
+    rounded reciprocal): the same scale and codes bit for bit. The row's only
+    other values are zeros (up = 0), so the scale is |h| / 7."""
+    g = np.arange(65536, dtype=np.uint16).view(np.float16)
+    g = g[np.isfinite(g)]
+    G, U = np.zeros((2, len(g), 16), np.float16), np.zeros((len(g), 16), np.float16)
+    G[:, :, 3], U[:, 3] = g, np.float16(1.37)
+    G[1, :, 4] = 100  # its up is 0
+    out = []
+    for Gi in G:
+        q = torch.empty((len(g), 8), dtype=torch.uint8, device=dev)
+        s = torch.empty((len(g),), dtype=torch.float32, device=dev)
+        p4q.p4q_swiglu_quant_expanded(torch.from_numpy(Gi).to(dev), torch.from_numpy(U).to(dev), q, s)
+        torch.cuda.synchronize()
+        assert p4q.p4q_device_status() == 0
+        out.append((q.cpu().numpy(), s.cpu().numpy().view(np.uint32)))
+    assert np.array_equal(out[0][1], out[1][1])
+    assert np.array_equal(out[0][0], out[1][0])
