@@ -47,20 +47,6 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// ---------------------------------------------------------------- 4-bit code of one value
-// clamp(round_half_even(fl32(h / s)), -8, 7) for a row scale s = fl32(a / 7),
-// |h| <= a, inv = fl32(1 / s): h * inv rounded to an integer by adding
-// 1.5 * 2^23 (whose bits then hold the integer in the low mantissa bits),
-// recomputed with the correctly rounded quotient near a .5 boundary (the two
-// quotients differ by less than 2^-19 there).
-__device__ __forceinline__ int q4_code(float h, float s, float inv) {
-  const float q = __fmul_rn(h, inv);
-  const float qm = __fadd_rn(q, 12582912.0f);
-  int r = __float_as_int(qm) - 0x4B400000;
-  if (fabsf(__fsub_rn(q, __fsub_rn(qm, 12582912.0f))) > 0.5f - 0x1p-17f) r = __float2int_rn(__fdiv_rn(h, s));
-  return max(-8, min(7, r));
-}
-
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -471,11 +457,6 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   return r;
 }
 
-// Arrive on an mbarrier of a cluster peer (or of this CTA) with cluster-scope release.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_saddr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_saddr) : "memory");
-}
-
 // Arrive on an mbarrier of a cluster peer (or of this CTA) with the default
 // (release, CTA-scope) semantics of mbarrier.arrive.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_saddr) {
@@ -484,44 +465,6 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_saddr) {
 
 __device__ __forceinline__ void st_shared_cluster_u32(uint32_t cluster_saddr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_saddr), "r"(v) : "memory");
-}
-
-// try_wait with cluster-scope acquire (the phase may have been completed by
-// arrivals from the peer CTA), sleeping up to hint_ns.
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity, uint32_t hint_ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(hint_ns)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait with cluster-scope acquire (see mbar_wait).
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                                  unsigned int* err) {
-  const uint32_t a = smem_u32(bar);
-  if (mbar_try_wait_cluster(a, parity, 0u)) return true;
-  const unsigned long long t0 = globaltimer();
-  while (true) {
-    if (mbar_try_wait_cluster(a, parity, 200000u)) return true;
-    if (*abort) return false;
-    if (globaltimer() - t0 > kWaitLimitNs) {
-      *abort = 1;
-      atomicOr(err, kErrTimeout);
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                                       unsigned int* err) {
-  int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_cluster(bar, parity, abort, err) ? 1 : 0;
-  return __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
 }
 
 // ---- tcgen05 for a CTA pair (cta_group::2): executed by one warp in each CTA

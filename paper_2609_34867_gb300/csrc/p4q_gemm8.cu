@@ -5,7 +5,7 @@
 // offset codes u = v + 8), for linears large enough to be tensor-bound.
 // Unpacking the nibbles inside the GEMM shares each SM's shared-memory path
 // and issue slots with the MMAs and halves the rate the tensor pipe gets;
-// here two streaming kernels first expand both packed operands into a
+// here a streaming kernel first expands both packed operands into a
 // caller workspace, one byte per code (the E4M3 byte u, exact), with the
 // per-row sums of u, and the GEMM's operands then reach shared memory by TMA
 // alone, already in the 128-byte-swizzled K-major layout the MMAs read.

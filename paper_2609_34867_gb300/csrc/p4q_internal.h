@@ -69,8 +69,6 @@ struct RowSource {
   const int32_t* idx = nullptr;    // [B, K] kept indices (gather mode)
   const uint16_t* text = nullptr;  // [B, T, L] (gather mode)
   int N = 0, K = 0, T = 0;         // gather mode sizes
-  const uint16_t* X2 = nullptr;    // dense rows split, split + 1, ... (the second sinks; dense mode)
-  int split = 0;
   // lets the next kernel launch before this one's wait (a linear that prefetches its
   // weights meanwhile); in the selector's chain that made calls 3% slower
   bool early = false;
@@ -86,10 +84,7 @@ struct RowSinks {
   int32_t* sum_u = nullptr;   // [rows] sum of u (with u)
 };
 
-// Rows at or past src.split (when src.X2 is set) come from X2 and go to
-// *out2, renumbered from 0: two row sets quantized by one launch.
-cudaError_t launch_quant_rows(const RowSource& src, int rows, int L, const RowSinks& out,
-                              cudaStream_t stream, const RowSinks* out2 = nullptr);
+cudaError_t launch_quant_rows(const RowSource& src, int rows, int L, const RowSinks& out, cudaStream_t stream);
 
 // Per-token quantizer of up to two column blocks of Y [M, ldy] fp16 whose
 // rows' abs-max is known (fp16 bit patterns rowmax [nblk, M], as the GEMM's

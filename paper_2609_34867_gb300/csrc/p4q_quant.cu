@@ -16,8 +16,7 @@
 //                             concepts.
 //   quant_rows_kernel         every other case (the fused gather of the
 //                             pruned sequence through the kept indices with
-//                             its fp16 copy, two row sets in one launch, other
-//                             row lengths): rows stream through shared memory,
+//                             its fp16 copy, few rows, other row lengths): rows stream through shared memory,
 //                             a group of G warps owning a ring of S row
 //                             buffers that its leader fills with bulk
 //                             asynchronous copies (cp.async.bulk, one mbarrier
@@ -55,7 +54,6 @@ constexpr uint32_t kInflightTarget = 48u * 1024u;  // bytes on their way per CTA
 constexpr int kSmemMax = 110 * 1024;
 
 __device__ __forceinline__ const uint16_t* row_ptr(const RowSource& src, int row, int L) {
-  if (src.X2 != nullptr && row >= src.split) return src.X2 + static_cast<size_t>(row - src.split) * L;
   if (src.idx == nullptr) return src.X + static_cast<size_t>(row) * (src.ldx > 0 ? src.ldx : L);
   const int per = src.K + src.T;
   const int b = row / per, r = row - b * per;
@@ -72,7 +70,7 @@ __device__ __forceinline__ const uint16_t* row_ptr(const RowSource& src, int row
 // in flight before the CTA exits.
 template <int G, bool NORM>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
-    quant_rows_kernel(RowSource src, int rows, int L, RowSinks out1, RowSinks out2, int S, uint32_t stage_bytes) {
+    quant_rows_kernel(RowSource src, int rows, int L, RowSinks out, int S, uint32_t stage_bytes) {
   constexpr int kGroups = kWarps / G;
   constexpr int kGroupThreads = 32 * G;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -114,9 +112,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   int consumed = 0;  // rows whose buffer this warp has seen complete
   for (int j = 0; j < mine; ++j) {
     const int st = j % S;
-    const bool second = src.X2 != nullptr && first + j * total >= src.split;
-    const RowSinks& out = second ? out2 : out1;
-    const int row = second ? first + j * total - src.split : first + j * total;  // row of its sinks
+    const int row = first + j * total;
     if (!failed) {
       failed = !mbar_wait_warp(&full[st], (j / S) & 1, abort, &g_quant_err);
       if (!failed) consumed = j + 1;
@@ -248,7 +244,7 @@ int sm_count() {
 }
 
 template <int G, bool NORM>
-cudaError_t launch_g(const RowSource& src, int rows, int L, const RowSinks& out, const RowSinks& out2, const Plan& p,
+cudaError_t launch_g(const RowSource& src, int rows, int L, const RowSinks& out, const Plan& p,
                      cudaStream_t stream) {
   static SmemLimit limit;
   const cudaError_t le = limit.allow(quant_rows_kernel<G, NORM>, kSmemMax);
@@ -258,19 +254,18 @@ cudaError_t launch_g(const RowSource& src, int rows, int L, const RowSinks& out,
                       3 * kWarps * 4 + kGroups * 4;
   const int need = (rows + kGroups - 1) / kGroups;
   const int grid = std::min(need, kCtasPerSm * sm_count());
-  return launch_pdl(quant_rows_kernel<G, NORM>, dim3(grid), dim3(kThreads), smem, stream, src, rows, L, out, out2,
-                    p.S, p.stage_bytes);
+  return launch_pdl(quant_rows_kernel<G, NORM>, dim3(grid), dim3(kThreads), smem, stream, src, rows, L, out, p.S,
+                    p.stage_bytes);
 }
 
 template <bool NORM>
-cudaError_t launch_norm(const RowSource& src, int rows, int L, const RowSinks& out, const RowSinks& out2,
-                        cudaStream_t stream) {
+cudaError_t launch_norm(const RowSource& src, int rows, int L, const RowSinks& out, cudaStream_t stream) {
   const Plan p = plan_for(L);
   switch (p.G) {
-    case 1: return launch_g<1, NORM>(src, rows, L, out, out2, p, stream);
-    case 2: return launch_g<2, NORM>(src, rows, L, out, out2, p, stream);
-    case 4: return launch_g<4, NORM>(src, rows, L, out, out2, p, stream);
-    default: return launch_g<8, NORM>(src, rows, L, out, out2, p, stream);
+    case 1: return launch_g<1, NORM>(src, rows, L, out, p, stream);
+    case 2: return launch_g<2, NORM>(src, rows, L, out, p, stream);
+    case 4: return launch_g<4, NORM>(src, rows, L, out, p, stream);
+    default: return launch_g<8, NORM>(src, rows, L, out, p, stream);
   }
 }
 
@@ -681,24 +676,18 @@ cudaError_t launch_select_token_quant(const uint16_t* V, int B, int N, int d, in
 }
 
 
-cudaError_t launch_quant_rows(const RowSource& src, int rows, int L, const RowSinks& out,
-                              cudaStream_t stream, const RowSinks* out2) {
+cudaError_t launch_quant_rows(const RowSource& src, int rows, int L, const RowSinks& out, cudaStream_t stream) {
   if (rows <= 0) return cudaSuccess;
-  if (src.X2 != nullptr && (out2 == nullptr || out2->codes == nullptr || out2->scale == nullptr || src.idx != nullptr ||
-                            src.ldx != 0 || (out.norm2 == nullptr) != (out2->norm2 == nullptr)))
-    return cudaErrorInvalidValue;
   // packed codes may be left out when the expanded ones are written
   if (out.scale == nullptr || (out.codes == nullptr && out.u == nullptr)) return cudaErrorInvalidValue;
-  const RowSinks& o2 = out2 ? *out2 : out;
   // dense rows of at most kRegRowMax elements, at least a wave of them: the
   // register-resident kernel (a few rows, e.g. the selector's concepts, run
   // faster in the chain on the ring kernel: measured 85 against 95 us per
   // 8 x 576 selector call)
-  if (rows >= kRegMinRows && src.X2 == nullptr && src.idx == nullptr && out.copy == nullptr && L % 256 == 0 &&
+  if (rows >= kRegMinRows && src.idx == nullptr && out.copy == nullptr && L % 256 == 0 &&
       L <= kRegRowMax && (out.u == nullptr) == (out.sum_u == nullptr))
     return out.norm2 ? launch_reg_norm<true>(src, rows, L, out, stream) : launch_reg_norm<false>(src, rows, L, out, stream);
-  return out.norm2 ? launch_norm<true>(src, rows, L, out, o2, stream)
-                   : launch_norm<false>(src, rows, L, out, o2, stream);
+  return out.norm2 ? launch_norm<true>(src, rows, L, out, stream) : launch_norm<false>(src, rows, L, out, stream);
 }
 
 unsigned int quant_read_and_clear_error() {
