@@ -43,7 +43,7 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 // its lifetime. Kernels therefore read with ordinary loads, which see everything
 // before pdl_wait(), and not through the read-only path (ld.global.nc, __ldg,
 // const __restrict__ parameters), which may return an older line of L1. (The
-// one exception, ldg_readonly16, states why its data is read-only.)
+// one use of ldg_readonly16 states why its data is read-only.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -209,7 +209,7 @@ cudaError_t launch_mr(const GemmArgs& g, cudaStream_t stream) {
 // the tensor-core kernel (p4q_fewrows.cu) is faster, which starts slower (3.7 -
 // 8 us for weights of any size up to 4 MB) and hardly depends on the rows. The
 // time here grows with the rows' staging and outputs and with the products; the
-// line's two terms are fitted to 1100 sizes (on average 0.8 % above the faster
+// line's two terms are fitted to 858 sizes (on average 0.8 % above the faster
 // kernel), us here / there: 3 x 1024 x 1024 (N x K) 2.2 / 4.8, 8 x 1024 x 4096 5.0 /
 // 5.3, 8 x 4096 x 1024 4.0 / 6.2, 4 x 4096 x 4096 6.7 / 6.8, 8 x 4096 x 4096 7.8 / 6.9, 3 x
 // 2048 x 8192 4.8 / 7.5, 8 x 512 x 11008 9.6 / 7.0, 8 x 8192 x 512 5.8 / 6.1.
