@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ __align__(8) uint64_t acc_full;          // MMA -> epilogue
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_word;
+  __shared__ int loads;                                // issued, for the give-up path
   __shared__ int sums[kMaxRowTile + 1];                // of x + 8, per activation row
   volatile int* abort_flag = &abort_word;
 
@@ -253,13 +254,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   if (warp == 0) {
     // ------------------------------------------------------------ packed weights by TMA
     if (lane == 0) {
-      bool ok = true;
       int s = 0, ph = 0;
       for (; issued < np; ++issued) {
-        if (!mbar_wait_spin(&empty[s], ph, abort_flag, &g_fewrows_err)) {
-          ok = false;
-          break;
-        }
+        if (!mbar_wait_spin(&empty[s], ph, abort_flag, &g_fewrows_err)) break;
         mbar_arrive_expect_tx(&full[s], kPairBytes);
         tma_load_3d(&tmW, &full[s], smem + s * kPairBytes, (kb0 + 2 * issued) * kBKP, n0, 0);
         if (++s == p.stages) {
@@ -267,13 +264,7 @@ __global__ void __launch_bounds__(kThreads, 2)
           ph ^= 1;
         }
       }
-      if (!ok) {
-        // leave no TMA load in flight into this CTA's shared memory
-        int fresh = 0;
-        for (int j = (issued > p.stages ? issued - p.stages : 0); j < issued; ++j)
-          mbar_wait(&full[j % p.stages], (j / p.stages) & 1, reinterpret_cast<volatile int*>(&fresh), &g_fewrows_err,
-                    100000000ull);
-      }
+      loads = issued;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMAs
@@ -365,6 +356,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
     }
     if (ok) ok = mbar_wait_all(&acc_full, 0, abort_flag, &g_fewrows_err);
+    else tmem_st_wait();  // given up: no store in flight when TMEM is released
     tc_fence_after();
     // this CTA's partial accumulators (exact integers) as [MP][128] floats in
     // place of the activations (every MMA that read them is complete)
@@ -429,6 +421,13 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   if (p.split > 1) cluster_sync();  // no CTA leaves while its partials are read
   else __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) {
+    // given up (whichever warp did): leave no TMA load in flight into this CTA's shared memory
+    int fresh = 0;
+    for (int j = (loads > p.stages ? loads - p.stages : 0); j < loads; ++j)
+      mbar_wait(&full[j % p.stages], (j / p.stages) & 1, reinterpret_cast<volatile int*>(&fresh), &g_fewrows_err,
+                100000000ull);
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmem);

@@ -1,8 +1,12 @@
-"""Stage 3 of the selector gives up (with an error status) when its phases run
+"""The give-up paths that no input reaches, checked on the source.
+
+Stage 3 of the selector gives up (with an error status) when its phases run
 past their limit or a bounded wait runs out. The block must leave its loop as
 one: threads that go on would wait at barriers for those that left, and the
-helper CTAs with them. No input reaches the limit, so the rule is checked on the
-source."""
+helper CTAs with them.
+
+The few-rows linear gives up when a wait of any of its warps runs out: its TMA
+loads in flight are then waited for, and a TMEM store before TMEM is released."""
 import os
 import re
 
@@ -21,3 +25,14 @@ def test_every_thread_leaves_at_the_same_phase():
     assert "for (int phase = 0;; ++phase)" in loop
     # no thread raises the flag by itself: only the bounded waits do, and those lie behind another barrier of the phase
     assert not re.search(r"abort_flag\s*=[^=]", kernel[kernel.index("phase_limit = "):])
+
+
+def test_few_rows_leaves_nothing_in_flight():
+    code = open(os.path.join(B.CSRC, "p4q_fewrows.cu")).read()
+    code = re.sub(r"//[^\n]*", "", code)
+    # the loads are waited for behind the barriers that every warp's abort precedes, not in the loading warp's own branch
+    tail = code[code.rindex("else __syncthreads();"):]
+    assert re.search(r"if \(threadIdx\.x == 0 && \*abort_flag\) \{[^}]*mbar_wait\(&full\[", tail)
+    # the unpack loop may be left between a TMEM store and its wait: waited for behind it
+    loop_end = code[code.index("tmem_st_16x256b_x8(ta"):]
+    assert re.search(r"if \(ok\) ok = mbar_wait_all\(&acc_full[^;]*;\s*else tmem_st_wait\(\);", loop_end)
